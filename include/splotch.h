@@ -313,8 +313,9 @@ int spl_mlp_nparam(void);   /* SPL_MLP_NPARAM */
 /* Network kernels on DEVICE buffers (stream: cudaStream_t or NULL).
  * forward:   d_y[b] = net(d_x[b]) for b < B (d_x row-major [B][32]).
  * loss_grad: d_grad = gradient of L = (1/B) sum_b (net(x_b) - t_b)^2 with
- *            respect to every parameter, d_loss (may be NULL) = L; allocates
- *            and frees its own scratch and waits for the stream.
+ *            respect to every parameter, d_loss (may be NULL) = L; waits for
+ *            the stream (its scratch is fixed per GPU; with more than four calls
+ *            at once the others allocate and free their own).
  * adam:      one Adam step (Kingma & Ba, Algorithm 1) on np parameters,
  *            step >= 1, moments d_m, d_v updated in place. */
 int spl_mlp_forward(const float *d_theta, const float *d_x, int64_t B, float *d_y, void *stream);

@@ -3,6 +3,7 @@
 //   raster+count -> count large -> scan -> [sync: size lists] -> scatter ->
 //   tile pass -> large pass -> (E=A epilogue)
 // all on one stream.
+#include <atomic>
 #include <cmath>
 #include <cstdio>
 #include <cstddef>
@@ -1217,19 +1218,53 @@ extern "C" int spl_mlp_forward(const float *d_theta, const float *d_x, int64_t B
     return cuda_status(cudaGetLastError());
 }
 
+// Scratch of spl_mlp_loss_grad: a few partial-gradient arrays per GPU, fixed when
+// the library is loaded (5.3 MB).  Allocating and freeing scratch in the call cost 120 us,
+// ten times its kernels.  Host threads claim a slot by an atomic flag;
+// a call that finds none free allocates.
+constexpr int kGradSlots = 4;
+static __device__ float spl_grad_scratch[kGradSlots][kGradBlocks * kGradRow];
+static std::atomic_flag g_grad_busy[kGradSlots] = {ATOMIC_FLAG_INIT, ATOMIC_FLAG_INIT,
+                                                   ATOMIC_FLAG_INIT, ATOMIC_FLAG_INIT};
+
+struct GradSlot {
+    int k = -1;
+    ~GradSlot() {
+        if (k >= 0) g_grad_busy[k].clear(std::memory_order_release);
+    }
+    // The array on the current device, or null.
+    float *get() {
+        for (int q = 0; q < kGradSlots && k < 0; ++q)
+            if (!g_grad_busy[q].test_and_set(std::memory_order_acquire)) k = q;
+        if (k < 0) return nullptr;
+        void *p = nullptr;
+        if (cudaGetSymbolAddress(&p, spl_grad_scratch) != cudaSuccess) {
+            cudaGetLastError();
+            return nullptr;
+        }
+        return static_cast<float *>(p) + (size_t)k * kGradBlocks * kGradRow;
+    }
+};
+
 extern "C" int spl_mlp_loss_grad(const float *d_theta, const float *d_x, const float *d_t, int64_t B,
                                  float *d_grad, float *d_loss, void *stream) {
     if (!d_theta || !d_grad || B < 1 || !d_x || !d_t) return SPL_EINVAL;
-    float *work = nullptr;
-    if (cudaMalloc((void **)&work, sizeof(float) * mlp_work_floats(B)) != cudaSuccess) {
-        cudaGetLastError();
-        return SPL_ENOMEM;
+    // the partial gradients: a slot of the fixed scratch when one is free (the
+    // call waits for the stream, so a slot is in use exactly while it is held)
+    GradSlot slot;
+    float *work = slot.get(), *own = nullptr;
+    if (!work) {
+        if (cudaMalloc((void **)&own, sizeof(float) * mlp_work_floats()) != cudaSuccess) {
+            cudaGetLastError();
+            return SPL_ENOMEM;
+        }
+        work = own;
     }
     cudaStream_t s = (cudaStream_t)stream;
     launch_mlp_loss_grad(d_theta, d_x, d_t, B, work, d_grad, d_loss, s);
     int rc = cuda_status(cudaGetLastError());
     if (rc == SPL_OK) rc = cuda_status(cudaStreamSynchronize(s));
-    cudaFree(work);
+    if (own) cudaFree(own);
     return rc;
 }
 
@@ -1246,7 +1281,7 @@ extern "C" int spl_mlp_train(const float *d_x, const float *d_t, int64_t B, floa
     if (!d_x || !d_t || B < 1 || !theta || steps < 0 || !(lr > 0.f)) return SPL_EINVAL;
     cudaStream_t s = (cudaStream_t)stream;
     float *buf = nullptr;
-    const size_t nf = 4 * (size_t)kNParam + (size_t)(steps + 1) + mlp_work_floats(B);
+    const size_t nf = 4 * (size_t)kNParam + (size_t)(steps + 1) + mlp_work_floats();
     if (cudaMalloc((void **)&buf, sizeof(float) * nf) != cudaSuccess) {
         cudaGetLastError();
         return SPL_ENOMEM;

@@ -242,7 +242,9 @@ void launch_mlp_loss_grad(const float *theta, const float *x, const float *t, in
                           float *work, float *grad, float *loss, cudaStream_t s);
 void launch_mlp_adam(float *theta, const float *grad, float *m, float *v, int64_t np, int64_t step,
                      float lr, float b1, float b2, float eps, cudaStream_t s);
-size_t mlp_work_floats(int64_t B);
+// One CTA's partial gradient and loss, and the CTAs of a gradient pass.
+constexpr int kGradRow = kNParam + 3, kGradBlocks = 152;
+size_t mlp_work_floats();
 // logc[k] = log(cycles[k]) (cycles clamped to >= 1).
 void launch_log_cycles(const long long *cycles, int64_t n, float *logc, cudaStream_t s);
 
