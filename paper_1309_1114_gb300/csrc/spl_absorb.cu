@@ -24,7 +24,7 @@ namespace spl {
 // (r^2 - dy^2) B + 1) (a point: A in its row, 2 for the clip), or, where a
 // lane's rows go two at a time, per row pair (A w_a, A w_b, clip_a, clip_b);
 // ssrc[2p], ssrc[2p + 1] = (E / A) per channel, each value twice (0 when
-// A = 0).  Thread (p, q) fills columns and rows (row pairs) q, q + 8, ... of
+// A = 0), then A.  Thread (p, q) fills columns and rows (row pairs) q, q + 8, ... of
 // particle p and tests row band q.
 template <int T>
 __device__ __forceinline__ void absorb_tabulate(const FrameConst &fc, const float4 *st0,
@@ -46,7 +46,7 @@ __device__ __forceinline__ void absorb_tabulate(const FrameConst &fc, const floa
         const float inv = A > 0.f ? 1.f / A : 0.f;
         const float e0 = r1.y * inv, e1 = r1.z * inv, e2 = r1.w * inv;
         ssrc[2 * p] = make_float4(e0, e0, e1, e1);
-        ssrc[2 * p + 1] = make_float4(e2, e2, 0.f, 0.f);
+        ssrc[2 * p + 1] = make_float4(e2, e2, A, 0.f);
     }
     // row table: per row (A w_y, clip term), or per row pair (A w_a, A w_b,
     // clip_a, clip_b) when rows go two at a time
@@ -156,6 +156,21 @@ __device__ __forceinline__ f32x2 one_minus_exp_neg2(f32x2 tau) {
     unpack2(sr, s0, s1);
     unpack2(ge, g0, g1);
     return pack2(t0 < 0.0625f ? s0 : g0, t1 < 0.0625f ? s1 : g1);
+}
+
+// The same where tau <= 1, two values at once: tau times the degree-5 Chebyshev
+// interpolant of (1 - exp(-tau)) / tau on [0, 1] (relative error 9.4e-8; with FP32
+// rounding at most 2.0e-7, 6.7e-8 rms).  A particle with 0 <= A <= 1 never exceeds it,
+// since its weights are at most 1, so that the choice is the same for the whole
+// warp; per pixel pair it saves the hardware exp2s, the branch's two compares and
+// selects and two packed operations.
+__device__ __forceinline__ f32x2 one_minus_exp_neg2_unit(f32x2 tau) {
+    f32x2 sr = fma2v(tau, pack2(-0.000912545391f, -0.000912545391f), pack2(0.00783736380f, 0.00783736380f));
+    sr = fma2v(tau, sr, pack2(-0.0414187630f, -0.0414187630f));
+    sr = fma2v(tau, sr, pack2(0.166609671f, 0.166609671f));
+    sr = fma2v(tau, sr, pack2(-0.499995160f, -0.499995160f));
+    sr = fma2v(tau, sr, pack2(0.999999933f, 0.999999933f));
+    return mul2(tau, sr);
 }
 
 template <int T>
@@ -273,6 +288,9 @@ __global__ void __launch_bounds__(kTileThreads, absorb_ctas<T>()) absorb_kernel(
                     const ulonglong2 s01 = sv[0], s2x = sv[1];
                     const ulonglong2 *rp =
                         reinterpret_cast<const ulonglong2 *>(&srow[0][0]) + p * (T / 2) + row0 / 2;
+                    float A, unused;
+                    unpack2(s2x.y, A, unused);
+                    const bool thin = A >= 0.f && A <= 1.f;
 #pragma unroll
                     for (int m = 0; m < RP; ++m) {
                         const ulonglong2 rv = rp[m];
@@ -283,7 +301,7 @@ __global__ void __launch_bounds__(kTileThreads, absorb_ctas<T>()) absorb_kernel(
                             const f32x2 clip =
                                 pack2(__saturatef(ca - dxb[k]), __saturatef(cb - dxb[k]));
                             const f32x2 tau = mul2(mul2(pack2(wx[k], wx[k]), clip), rv.x);
-                            const f32x2 f = mul2(Tr2[m][k], one_minus_exp_neg2(tau));
+                            const f32x2 f = mul2(Tr2[m][k], thin ? one_minus_exp_neg2_unit(tau) : one_minus_exp_neg2(tau));
                             fma2(C2[m][k][0], f, s01.x);
                             fma2(C2[m][k][1], f, s01.y);
                             fma2(C2[m][k][2], f, s2x.x);
@@ -342,34 +360,56 @@ __global__ void __launch_bounds__(kTileThreads, absorb_ctas<T>()) absorb_kernel(
     }
 }
 
-// Tiles cut into several items: compose the items' partials in list order.
+// Tiles cut into several items: compose the items' partials in list order.  A CTA
+// takes 32 pixels of a tile; each of its eight warps composes an eighth of the
+// items, and the eighths are composed in order (the composition is associative).
+// Bound by the partials' traffic (16 B per pixel and item): a crowded tile has
+// hundreds of items, and one thread per pixel running through all of them in four
+// passes of a single CTA per tile was a chain of loads (597 us for the clustered
+// 10M / 1024^2 frame; now COMBINE_US).
 template <int T>
 __global__ void __launch_bounds__(256) absorb_combine_kernel(Views vs, const int *item_offsets,
                                                              const float4 *partial,
                                                              float *const *images) {
-    for (int g = blockIdx.x; g < vs.total_tiles; g += gridDim.x) {
-        const int i0 = item_offsets[g], i1 = item_offsets[g + 1];
-        if (i1 - i0 < 2) continue;
-        const int view = view_of_tile(vs.fcs, vs.nviews, g);
-        const FrameConst &fc = vs.fcs[view];
-        const int tile = g - fc.tile_base;
-        const int x0 = (tile % fc.ntx) * T, y0 = (tile / fc.ntx) * T;
-        for (int px = threadIdx.x; px < T * T; px += blockDim.x) {
-            const int row = px / T, cx = px % T;
-            if (y0 + row >= fc.height || x0 + cx >= fc.width) continue;
-            float c0 = 0.f, c1 = 0.f, c2 = 0.f, tr = 1.f;
-            for (int it = i0; it < i1; ++it) {
-                const float4 v = partial[(size_t)it * (T * T) + px];
+    constexpr int GROUPS = T * T / 32;
+    __shared__ float4 part[8][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (long long u = blockIdx.x; u < (long long)vs.total_tiles * GROUPS; u += gridDim.x) {
+        const int g = (int)(u / GROUPS), px = (int)(u % GROUPS) * 32 + lane;
+        const int i0 = item_offsets[g], n = item_offsets[g + 1] - i0;
+        if (n < 2) continue;                       // the same for the whole CTA
+        const int a = i0 + (int)((long long)n * warp / 8), b = i0 + (int)((long long)n * (warp + 1) / 8);
+        float c0 = 0.f, c1 = 0.f, c2 = 0.f, tr = 1.f;
+#pragma unroll 4
+        for (int it = a; it < b; ++it) {
+            const float4 v = partial[(size_t)it * (T * T) + px];
+            c0 = fmaf(tr, v.x, c0);
+            c1 = fmaf(tr, v.y, c1);
+            c2 = fmaf(tr, v.z, c2);
+            tr *= v.w;
+        }
+        part[warp][lane] = make_float4(c0, c1, c2, tr);
+        __syncthreads();
+        if (warp == 0) {
+            for (int k = 1; k < 8; ++k) {
+                const float4 v = part[k][lane];
                 c0 = fmaf(tr, v.x, c0);
                 c1 = fmaf(tr, v.y, c1);
                 c2 = fmaf(tr, v.z, c2);
                 tr *= v.w;
             }
-            float *dst = images[view] + 3 * ((int64_t)(y0 + row) * fc.width + x0 + cx);
-            dst[0] = c0;
-            dst[1] = c1;
-            dst[2] = c2;
+            const int view = view_of_tile(vs.fcs, vs.nviews, g);
+            const FrameConst &fc = vs.fcs[view];
+            const int tile = g - fc.tile_base;
+            const int x = (tile % fc.ntx) * T + px % T, y = (tile / fc.ntx) * T + px / T;
+            if (x < fc.width && y < fc.height) {
+                float *dst = images[view] + 3 * ((int64_t)y * fc.width + x);
+                dst[0] = c0;
+                dst[1] = c1;
+                dst[2] = c2;
+            }
         }
+        __syncthreads();
     }
 }
 
@@ -379,7 +419,8 @@ static void launch_absorb_t(const Views &vs, const TileArgs &a, const int *item_
     constexpr size_t bytes = absorb_smem_bytes<T>();
     absorb_kernel<T><<<sms * absorb_ctas<T>(), kTileThreads, bytes, s>>>(vs, a);
     ++g_launches;
-    const int grid = vs.total_tiles < sms * 8 ? vs.total_tiles : sms * 8;
+    const long long units = (long long)vs.total_tiles * (T * T / 32);
+    const int grid = (int)(units < sms * 8 ? units : sms * 8);
     if (grid > 0) {
         absorb_combine_kernel<T><<<grid, 256, 0, s>>>(vs, item_offsets, a.partial, a.images);
         ++g_launches;

@@ -1,0 +1,42 @@
+"""General absorption where its kernels branch: particles with A on both sides of
+1 (the two forms of 1 - exp(-tau)), negative and zero A left out, and tiles cut
+into 2, 7, 8, 9 and more segments (the composition takes eighths of them), against the FP64
+oracle within the mode's bar (1e-4)."""
+import os
+
+import numpy as np
+import pytest
+
+import oracle
+from paper_1309_1114_gb300 import scenes
+from tests._metrics import rel_pixel_error
+from tests.test_gpu_parity import gpu_render
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def rnd():
+    import torch
+    assert torch.cuda.is_available()
+    from paper_1309_1114_gb300.splotch import Renderer
+    r = Renderer(0)
+    yield r
+    r.close()
+
+
+@pytest.mark.parametrize("tile", [16, 32, 64])
+@pytest.mark.parametrize("n,scale", [(900, 1.0), (1500, 2.5), (7100, 0.05), (8300, 1.0), (9300, 0.3)])
+def test_one_crowded_tile(rnd, tile, n, scale):
+    import torch
+    rng = np.random.default_rng(n)
+    # every particle reaches the middle tile: lists of n entries, cut every 1024
+    p = {"x": rng.normal(0.5, 0.002, n), "y": rng.normal(0.5, 0.002, n), "z": rng.random(n),
+         "h": np.exp(rng.uniform(-6.0, -4.5, n)), "I": scale * rng.random(n) ** 4, "s": rng.random(n)}
+    p = {k: v.astype(np.float32) for k, v in p.items()}
+    cam = scenes.camera(3 * 64, 2 * 64 + 5)
+    g = gpu_render(rnd, torch, p, scenes.ramp_palette(), cam, mode=2, tile_px=tile)
+    par = {"mode": 2}
+    o = oracle.render(p, scenes.ramp_palette(), cam, par, nthreads=os.cpu_count() or 1)
+    B, _ = oracle.ambiguity(p, scenes.ramp_palette(), cam, par)
+    assert rel_pixel_error(g, o, B) <= 1e-4
