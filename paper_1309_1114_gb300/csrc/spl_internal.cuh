@@ -88,16 +88,18 @@ struct DevStats {
 // A work item of the persistent tile / large passes: a tile (global index
 // over the batch) and a range of one of its lists, or every list of a tile
 // light enough to be done by one CTA, which then stores its pixels instead of
-// adding them.  lv packs the view (high bits) and the list (low 8 bits, 0xFF
-// for "every list").
+// adding them (its range is the tile's medium list).  lv packs the view (high
+// bits), whether the item is its tile's only large item (kSole), and the list
+// (low 7 bits, kAllLists for "every list").
 struct WorkItem {
     int tile, lv;
     long long start, end;
 };
-constexpr int kAllLists = 0xFF;
+constexpr int kAllLists = 0x7F, kSole = 0x80;
 __host__ __device__ inline int item_view(const WorkItem &w) { return w.lv >> 8; }
+__host__ __device__ inline bool item_sole(const WorkItem &w) { return (w.lv & kSole) != 0; }
 __host__ __device__ inline int item_list(const WorkItem &w) {
-    return (w.lv & 0xFF) == kAllLists ? -1 : (w.lv & 0xFF);
+    return (w.lv & kAllLists) == kAllLists ? -1 : (w.lv & kAllLists);
 }
 
 // Largest list segment one work item takes (per list), so that a crowded

@@ -643,7 +643,9 @@ __global__ void fill_items_kernel(Views vs, const long long *off, const int *iof
         int w = ioff[g];
         const int nw = ioff[g + 1] - w;
         if (nw == 1) {
-            if (lane == 0) put_item(items, cap, w, {g, (v << 8) | kAllLists, 0, 0}, st);
+            if (lane == 0)
+                put_item(items, cap, w, {g, (v << 8) | kAllLists, off[sb + L_MEDIUM * nt + t],
+                                         off[sb + L_MEDIUM * nt + t + 1]}, st);
         } else if (nw > 1) {
             for (int l = 0; l < L_LARGE; ++l) {
                 const long long b = off[sb + l * nt + t], e = off[sb + l * nt + t + 1];
@@ -661,7 +663,8 @@ __global__ void fill_items_kernel(Views vs, const long long *off, const int *iof
         for (int k = lane; k < ns; k += 32) {
             const long long kb = b + (long long)k * kSegLarge;
             put_item(items, cap, wl + k,
-                     {g, (v << 8) | L_LARGE, kb, kb + kSegLarge < e ? kb + kSegLarge : e}, st);
+                     {g, (v << 8) | (ns == 1 ? kSole : 0) | L_LARGE, kb,
+                      kb + kSegLarge < e ? kb + kSegLarge : e}, st);
         }
     }
 }
