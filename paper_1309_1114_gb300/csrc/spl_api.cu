@@ -654,6 +654,14 @@ static int size_item_buffers(spl_ctx *c) {
     return SPL_OK;
 }
 
+// Items recorded as training samples, or put in an order by their predicted cost, keep
+// the full segments; so does the absorption mode, whose split tiles need a partial
+// tile each.
+static int seg_sms(const spl_ctx *c) {
+    const bool plain = !c->recording && c->par.sched == SPL_SCHED_NONE && c->par.mode != SPL_MODE_ABSORB;
+    return plain ? c->sms : 0;
+}
+
 // Stage 1: constants to the device, rasterise every view, count and scan the
 // list slots and the work items.
 static void enqueue_binning(spl_ctx *c, const Views &vs, cudaStream_t s) {
@@ -700,7 +708,7 @@ static void enqueue_binning(spl_ctx *c, const Views &vs, cudaStream_t s) {
     launch_count_large(vs, ba, c->sms, s);
     launch_slot_offsets(NLIST * vs.total_tiles, c->counts.p, c->ovf.p, c->offsets.p, c->cursor.p,
                         &c->dstats.p->slot_total, s);
-    launch_item_counts(vs, c->offsets.p, c->item_counts.p, c->dstats.p, s);
+    launch_item_counts(vs, c->offsets.p, c->item_counts.p, c->dstats.p, seg_sms(c), s);
     launch_scan(2 * vs.total_tiles, c->item_counts.p, c->item_offsets.p, nullptr, 2,
                 c->dstats.p->item_totals, s);
 }
@@ -723,7 +731,7 @@ static void enqueue_lists(spl_ctx *c, const Views &vs, cudaStream_t s) {
     ba.st = c->dstats.p;
     launch_scatter(vs, ba, c->sms, s);
     launch_fill_items(vs, c->offsets.p, c->item_offsets.p, c->items.p, (int)c->items.cap,
-                      c->dstats.p, s);
+                      c->dstats.p, seg_sms(c), s);
 }
 
 // Stage 3: schedule the work items, the tile and large passes, the epilogue.
@@ -1550,7 +1558,10 @@ extern "C" int spl_render_noalloc(const spl_particles *p, const spl_camera *cam,
     ba.st = dst;
     launch_count_large(vs, ba, sms, s);
     launch_slot_offsets(NLIST * fc.ntiles, counts, ovf, offsets, cursor, &dst->slot_total, s);
-    launch_item_counts(vs, offsets, item_counts, dst, s);
+    // on images of up to 4096 tiles: the extra items (at most 8 per CTA of the passes
+    // and list) then stay far below the fixed limit
+    const int seg = fc.ntiles <= 4096 ? sms : 0;
+    launch_item_counts(vs, offsets, item_counts, dst, seg, s);
     launch_scan(2 * fc.ntiles, item_counts, item_offsets, nullptr, 2, dst->item_totals, s);
     SPL_CUDA(cudaGetLastError());
     DevStats h;
@@ -1569,7 +1580,7 @@ extern "C" int spl_render_noalloc(const spl_particles *p, const spl_camera *cam,
     ba.entries = entries;
     ba.entries_cap = kNaMaxEntries;
     launch_scatter(vs, ba, sms, s);
-    launch_fill_items(vs, offsets, item_offsets, items, kNaMaxItems, dst, s);
+    launch_fill_items(vs, offsets, item_offsets, items, kNaMaxItems, dst, seg, s);
     TileArgs ta{};
     ta.recs = recs;
     ta.offsets = offsets;

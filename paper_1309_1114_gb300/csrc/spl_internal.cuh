@@ -105,6 +105,14 @@ __host__ __device__ inline int item_list(const WorkItem &w) {
 // Largest list segment one work item takes (per list), so that a crowded
 // tile (a halo core holding 1e5-1e6 particles) is spread over many CTAs.
 constexpr int kSegPoint = 8192, kSegSmall = 2048, kSegMedium = 1024, kSegLarge = 512;
+// A frame with less than two such segments for each CTA of the persistent passes
+// leaves most of them idle (200k particles on 256^2: 64 tiles, one item each, tile
+// pass 0.064 ms).  There the segments shrink with the frame's entries, down to
+// 1/8 of the above: two batches of the tile pass (0.047 ms; 1/4 and 1/16 within 5 %).
+constexpr int kSegShrink = 8;
+struct Segs {
+    int len[NLIST];
+};
 
 // Binning CTAs: each takes kChunk consecutive particles and aggregates their
 // list slots in a shared-memory hash table of kHash slots, which the scatter
@@ -195,10 +203,11 @@ void launch_scan(int m, const int *in, long long *out, long long *cursor, int ns
                  long long *seg_totals, cudaStream_t s);
 void launch_scan(int m, const int *in, int *out, int *cursor, int nseg, int *seg_totals,
                  cudaStream_t s);
+// sms > 0: segments shrink on small frames (see kSegShrink); 0: full segments.
 void launch_item_counts(const Views &v, const long long *offsets, int *item_counts, DevStats *st,
-                        cudaStream_t s);
+                        int sms, cudaStream_t s);
 void launch_fill_items(const Views &v, const long long *offsets, const int *item_offsets,
-                       WorkItem *items, int items_cap, DevStats *st, cudaStream_t s);
+                       WorkItem *items, int items_cap, DevStats *st, int sms, cudaStream_t s);
 void launch_scatter(const Views &v, const BinArgs &a, int sms, cudaStream_t s);
 void launch_tile_pass(const Views &v, const TileArgs &a, int sms, cudaStream_t s);
 void launch_large_pass(const Views &v, const TileArgs &a, int sms, cudaStream_t s);

@@ -576,16 +576,51 @@ void launch_slot_offsets(int m, int *counts, int *ovf, long long *offsets, long 
 
 // ---------------------------------------------------------------------------
 // Work items: a light tile is one item (all its lists, pixels stored); a
-// crowded tile is cut into segments of at most kSeg* entries per list, each
-// its own item (pixels added).  Large-list entries always form separate
+// crowded tile is cut into segments of at most kSeg* entries per list (fewer on
+// small frames), each its own item (pixels added).  Large-list entries always form separate
 // items of the large pass.  item_counts = [tile-pass items | large items].
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ int div_up(int a, int b) { return (a + b - 1) / b; }
 
-__global__ void item_count_kernel(Views vs, const long long *off, int *item_counts, DevStats *st) {
-    __shared__ int lt[NLIST];
-    if (threadIdx.x < NLIST) lt[threadIdx.x] = 0;
+// Segment lengths of this frame, the same in every CTA that asks (the lists' totals
+// are differences of their first and last offsets, summed over the views).  The
+// weights are the lists' cost per entry in the tile pass, in medium entries.
+__device__ __forceinline__ void frame_segs(const Views &vs, const long long *off, int sms, Segs *segs,
+                                           unsigned long long *tot) {
+    if (threadIdx.x < NLIST) tot[threadIdx.x] = 0ull;
     __syncthreads();
+    if (sms > 0)
+        for (int k = threadIdx.x; k < vs.nviews * NLIST; k += blockDim.x) {
+            const FrameConst &fc = vs.fcs[k / NLIST];
+            const int l = k % NLIST, b = fc.slot_base + l * fc.ntiles;
+            atomicAdd(&tot[l], (unsigned long long)(off[b + fc.ntiles] - off[b]));
+        }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        const int full[NLIST] = {kSegPoint, kSegSmall, kSegMedium, kSegLarge};
+        // CTAs of the passes: 4 per SM; two segments each
+        const unsigned long long work = tot[L_MEDIUM] + tot[L_SMALL] / 8 + tot[L_POINT] / 64;
+        for (int l = 0; l < NLIST; ++l) {
+            const int whole = l == L_LARGE ? kSegLarge : kSegMedium;
+            long long len = whole;
+            if (sms > 0) {
+                len = (long long)((l == L_LARGE ? tot[L_LARGE] : work) / (unsigned long long)(8 * sms));
+                len = (len + 63) / 64 * 64;
+                len = len < whole / kSegShrink ? whole / kSegShrink : (len > whole ? whole : len);
+            }
+            segs->len[l] = (int)(full[l] / whole * len);
+        }
+    }
+    __syncthreads();
+}
+
+__global__ void item_count_kernel(Views vs, const long long *off, int *item_counts, DevStats *st,
+                                  int sms) {
+    __shared__ int lt[NLIST];
+    __shared__ Segs segs;
+    __shared__ unsigned long long tots[NLIST];
+    if (threadIdx.x < NLIST) lt[threadIdx.x] = 0;
+    frame_segs(vs, off, sms, &segs, tots);
     const int T = vs.total_tiles;
     int tot[NLIST] = {0, 0, 0, 0};
     for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < T; g += gridDim.x * blockDim.x) {
@@ -598,13 +633,14 @@ __global__ void item_count_kernel(Views vs, const long long *off, int *item_coun
         tot[0] += cp; tot[1] += cs; tot[2] += cm; tot[3] += cl;
         int n = 0;
         if (cp + cs + cm > 0) {
-            if (cp <= kSegPoint && cs <= kSegSmall && cm <= kSegMedium)
+            if (cp <= segs.len[L_POINT] && cs <= segs.len[L_SMALL] && cm <= segs.len[L_MEDIUM])
                 n = 1;
             else
-                n = div_up(cp, kSegPoint) + div_up(cs, kSegSmall) + div_up(cm, kSegMedium);
+                n = div_up(cp, segs.len[L_POINT]) + div_up(cs, segs.len[L_SMALL]) +
+                    div_up(cm, segs.len[L_MEDIUM]);
         }
         item_counts[g] = n;
-        item_counts[T + g] = div_up(cl, kSegLarge);
+        item_counts[T + g] = div_up(cl, segs.len[L_LARGE]);
     }
     for (int l = 0; l < NLIST; ++l) {
         const int v = __reduce_add_sync(0xffffffffu, tot[l]);
@@ -615,9 +651,9 @@ __global__ void item_count_kernel(Views vs, const long long *off, int *item_coun
 }
 
 void launch_item_counts(const Views &vs, const long long *offsets, int *item_counts, DevStats *st,
-                        cudaStream_t s) {
+                        int sms, cudaStream_t s) {
     const int blocks = (vs.total_tiles + 255) / 256;
-    item_count_kernel<<<blocks, 256, 0, s>>>(vs, offsets, item_counts, st);
+    item_count_kernel<<<blocks, 256, 0, s>>>(vs, offsets, item_counts, st, sms);
     ++g_launches;
 }
 
@@ -631,9 +667,12 @@ __device__ __forceinline__ void put_item(WorkItem *items, int cap, int pos, Work
 // One warp per tile: the lanes write the tile's segments side by side (a
 // crowded tile has hundreds), in the same order as one thread would.
 __global__ void fill_items_kernel(Views vs, const long long *off, const int *ioff, WorkItem *items,
-                                  int cap, DevStats *st) {
+                                  int cap, DevStats *st, int sms) {
     const int T = vs.total_tiles;
-    const int seg[NLIST] = {kSegPoint, kSegSmall, kSegMedium, kSegLarge};
+    __shared__ Segs segs;
+    __shared__ unsigned long long tots[NLIST];
+    frame_segs(vs, off, sms, &segs, tots);
+    const int *seg = segs.len;
     const int lane = threadIdx.x & 31;
     const int warps = (gridDim.x * blockDim.x) >> 5;
     for (int g = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; g < T; g += warps) {
@@ -659,20 +698,20 @@ __global__ void fill_items_kernel(Views vs, const long long *off, const int *iof
         }
         const int wl = ioff[T + g];
         const long long b = off[sb + L_LARGE * nt + t], e = off[sb + L_LARGE * nt + t + 1];
-        const int ns = (int)((e - b + kSegLarge - 1) / kSegLarge);
+        const int sl = seg[L_LARGE], ns = (int)((e - b + sl - 1) / sl);
         for (int k = lane; k < ns; k += 32) {
-            const long long kb = b + (long long)k * kSegLarge;
+            const long long kb = b + (long long)k * sl;
             put_item(items, cap, wl + k,
                      {g, (v << 8) | (ns == 1 ? kSole : 0) | L_LARGE, kb,
-                      kb + kSegLarge < e ? kb + kSegLarge : e}, st);
+                      kb + sl < e ? kb + sl : e}, st);
         }
     }
 }
 
 void launch_fill_items(const Views &vs, const long long *offsets, const int *item_offsets,
-                       WorkItem *items, int items_cap, DevStats *st, cudaStream_t s) {
+                       WorkItem *items, int items_cap, DevStats *st, int sms, cudaStream_t s) {
     const int blocks = (vs.total_tiles + 7) / 8;     // 8 warps of 256 threads, a warp per tile
-    fill_items_kernel<<<blocks, 256, 0, s>>>(vs, offsets, item_offsets, items, items_cap, st);
+    fill_items_kernel<<<blocks, 256, 0, s>>>(vs, offsets, item_offsets, items, items_cap, st, sms);
     ++g_launches;
 }
 
