@@ -740,6 +740,7 @@ static void enqueue_passes(spl_ctx *c, const Views &vs, bool large_pass, cudaStr
     ta.recs = c->recs.p;
     ta.offsets = c->offsets.p;
     ta.entries = c->entries.p;
+    ta.entries_cap = (long long)c->entries.cap;
     ta.items = c->items.p;
     ta.items_cap = (int)c->items.cap;
     ta.images = c->d_images.p;
@@ -1585,6 +1586,7 @@ extern "C" int spl_render_noalloc(const spl_particles *p, const spl_camera *cam,
     ta.recs = recs;
     ta.offsets = offsets;
     ta.entries = entries;
+    ta.entries_cap = kNaMaxEntries;
     ta.items = items;
     ta.items_cap = kNaMaxItems;
     ta.images = d_img;

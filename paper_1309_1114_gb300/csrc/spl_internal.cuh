@@ -171,6 +171,7 @@ struct TileArgs {
     const Rec *recs;
     const long long *offsets;  // list slots of all views, + 1 (64-bit list positions)
     const unsigned *entries;
+    long long entries_cap;     // a replayed graph's lists may end beyond it (then flagged)
     const WorkItem *items;
     int items_cap;
     float *const *images;      // device array: one image per view

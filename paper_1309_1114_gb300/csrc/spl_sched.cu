@@ -63,6 +63,8 @@ __global__ void __launch_bounds__(256) item_features_kernel(Views vs, TileArgs a
                 b = w.start;
                 e = w.end;
             }
+            b = min(b, a.entries_cap);
+            e = min(e, a.entries_cap);
             total += (int)(e - b);
             long long stride = 1;
             if (max_sample > 0 && e - b > max_sample) stride = (e - b + max_sample - 1) / max_sample;

@@ -622,7 +622,8 @@ __global__ void __launch_bounds__(kTileThreads, min_ctas<T>()) item_kernel(Views
         if (list < 0 && tid < 4)
             s_range[tid] = a.offsets[fc.slot_base + (tid < 2 ? L_POINT : L_SMALL) * fc.ntiles + tile + (tid & 1)];
         const bool mine = list < 0 || list >= L_MEDIUM;   // medium (tile pass) or large (large pass)
-        const long long lb2 = mine ? w.start : 0, le2 = mine ? w.end : 0;
+        const long long cap = a.entries_cap;              // never past the entries written
+        const long long lb2 = mine ? min(w.start, cap) : 0, le2 = mine ? min(w.end, cap) : 0;
         const int col = (warp % S::NBX) * S::BW + (lane % S::LW) * S::CMUL;
         const int row0 = (warp / S::NBX) * S::BH + (lane / S::LW) * S::RPL;
         Acc<T> acc;
@@ -690,12 +691,12 @@ __global__ void __launch_bounds__(kTileThreads, min_ctas<T>()) item_kernel(Views
         long long lb0 = 0, le0 = 0, lb1 = 0, le1 = 0;
         if (list < 0) {
             if (lb2 >= le2) __syncthreads();   // s_range (the batches' barriers otherwise)
-            lb0 = s_range[0]; le0 = s_range[1];
-            lb1 = s_range[2]; le1 = s_range[3];
+            lb0 = min(s_range[0], cap); le0 = min(s_range[1], cap);
+            lb1 = min(s_range[2], cap); le1 = min(s_range[3], cap);
         } else if (list == L_POINT) {
-            lb0 = w.start; le0 = w.end;
+            lb0 = min(w.start, cap); le0 = min(w.end, cap);
         } else if (list == L_SMALL) {
-            lb1 = w.start; le1 = w.end;
+            lb1 = min(w.start, cap); le1 = min(w.end, cap);
         }
         const bool shared_tile = le0 > lb0 || le1 > lb1;
         if (shared_tile) {

@@ -62,3 +62,29 @@ def test_recorded_items_keep_full_segments(rnd):
         rnd.set_recording(False)
     # 900 entries per tile at most: one item each
     assert n == 4
+
+
+@pytest.mark.parametrize("grow", [4.0, 40.0])
+def test_replayed_lists_that_outgrow_their_buffers(grow):
+    """The passes of a replayed graph must not read entries past the buffer their lists
+    outgrew (a fresh context: nothing larger was rendered in it before)."""
+    import torch
+    from paper_1309_1114_gb300.splotch import Renderer
+    p = scenes.make("uniform", n=30_000).parts
+    big = dict(p, h=(p["h"] * np.float32(grow)))
+    cams = [scenes.camera(160, 120, azimuth_deg=a) for a in (0.0, 120.0)]
+    r = Renderer(0)
+    try:
+        r.set_colormap(scenes.ramp_palette())
+        r.set_params(r_large=20.0)
+        imgs = [torch.empty((120, 160, 3), device="cuda") for _ in cams]
+        for parts in (p, p, big):            # eager, replay, a replay that overflows
+            r.load(parts)
+            r.render_batch(cams, imgs)
+        torch.cuda.synchronize()
+        for cam, im in zip(cams, imgs):
+            o = oracle.render(big, scenes.ramp_palette(), cam, {}, nthreads=os.cpu_count() or 1)
+            B, _ = oracle.ambiguity(big, scenes.ramp_palette(), cam, {})
+            assert rel_pixel_error(im.cpu().numpy().astype(np.float64), o, B) <= 1e-4
+    finally:
+        r.close()
