@@ -102,6 +102,7 @@ struct spl_ctx {
     DevBuf<long long> offsets, cursor;
     DevBuf<unsigned> large_ids, entries;
     DevBuf<int> item_counts, item_offsets;
+    DevBuf<long long> slot_part;
     DevBuf<WorkItem> items;
     DevBuf<DevStats> dstats;
     DevBuf<float> host_img_scratch;
@@ -282,6 +283,7 @@ extern "C" int spl_destroy(spl_ctx *c) {
     c->ovf.release(); c->ctab.release();
     c->large_ids.release(); c->entries.release(); c->dstats.release();
     c->item_counts.release(); c->item_offsets.release(); c->items.release();
+    c->slot_part.release();
     c->host_img_scratch.release();
     c->d_fcs.release(); c->d_images.release();
     c->feat.release(); c->cost.release(); c->theta.release(); c->heur.release();
@@ -631,6 +633,7 @@ static int prepare_views(spl_ctx *c, const spl_camera *cams, int V, float *const
     SPL_TRY(grow(c, c->cursor, (size_t)NLIST * tiles));
     SPL_TRY(grow(c, c->item_counts, (size_t)2 * tiles));
     SPL_TRY(grow(c, c->item_offsets, (size_t)2 * tiles + 1));
+    SPL_TRY(grow(c, c->slot_part, slot_parts(tiles)));
     SPL_TRY(grow(c, c->entries, 16));
     SPL_TRY(grow(c, c->items, 16));
     SPL_TRY(grow(c, c->d_fcs, kMaxViews));
@@ -664,12 +667,25 @@ static int seg_sms(const spl_ctx *c) {
 
 // Stage 1: constants to the device, rasterise every view, count and scan the
 // list slots and the work items.
-static void enqueue_binning(spl_ctx *c, const Views &vs, cudaStream_t s) {
-    cudaMemcpyAsync(c->d_fcs.p, c->h_fcs, sizeof(FrameConst) * vs.nviews, cudaMemcpyHostToDevice, s);
-    cudaMemcpyAsync(c->d_images.p, c->h_images, sizeof(float *) * vs.nviews, cudaMemcpyHostToDevice, s);
-    cudaMemsetAsync(c->counts.p, 0, sizeof(int) * NLIST * vs.total_tiles, s);
-    cudaMemsetAsync(c->ovf.p, 0, sizeof(int) * NLIST * vs.total_tiles, s);
-    cudaMemsetAsync(c->dstats.p, 0, offsetof(DevStats, err), s);
+// `captured`: the launches go into a graph, whose replays read the constants from the
+// pinned staging; otherwise a single view's travel as launch arguments.
+static void enqueue_binning(spl_ctx *c, const Views &vs, bool captured, cudaStream_t s) {
+    SetupArgs sa{};
+    sa.counts = c->counts.p;
+    sa.ovf = c->ovf.p;
+    sa.slots = NLIST * vs.total_tiles;
+    sa.st = c->dstats.p;
+    if (captured || vs.nviews > 1) {
+        cudaMemcpyAsync(c->d_fcs.p, c->h_fcs, sizeof(FrameConst) * vs.nviews, cudaMemcpyHostToDevice, s);
+        cudaMemcpyAsync(c->d_images.p, c->h_images, sizeof(float *) * vs.nviews, cudaMemcpyHostToDevice,
+                        s);
+    } else {
+        sa.fc = c->h_fcs[0];
+        sa.image = c->h_images[0];
+        sa.fcs = c->d_fcs.p;
+        sa.images = c->d_images.p;
+    }
+    launch_setup(sa, c->sms, s);
     RasterArgs ra{};
     ra.n = src_n(c);
     if (c->streaming) {
@@ -706,18 +722,15 @@ static void enqueue_binning(spl_ctx *c, const Views &vs, cudaStream_t s) {
     ba.cursor = c->cursor.p;
     ba.st = c->dstats.p;
     launch_count_large(vs, ba, c->sms, s);
-    launch_slot_offsets(NLIST * vs.total_tiles, c->counts.p, c->ovf.p, c->offsets.p, c->cursor.p,
-                        &c->dstats.p->slot_total, s);
-    launch_item_counts(vs, c->offsets.p, c->item_counts.p, c->dstats.p, seg_sms(c), s);
-    launch_scan(2 * vs.total_tiles, c->item_counts.p, c->item_offsets.p, nullptr, 2,
-                c->dstats.p->item_totals, s);
+    const SlotArgs la{c->counts.p,      c->ovf.p,         c->offsets.p,      c->cursor.p,
+                      c->slot_part.p,   c->item_counts.p, c->item_offsets.p, c->dstats.p};
+    launch_slots(vs, la, seg_sms(c), s);
 }
 
 // Stage 2: clear the images and fill the tile lists and work items into the
 // current capacities (the kernels check them and flag an overflow instead of
 // writing past the end).
 static void enqueue_lists(spl_ctx *c, const Views &vs, cudaStream_t s) {
-    if (!c->accumulate) launch_zero_images(vs, c->d_images.p, c->sms, s);
     BinArgs ba{};
     ba.recs = c->recs.p;
     ba.large_ids = c->large_ids.p;
@@ -729,9 +742,8 @@ static void enqueue_lists(spl_ctx *c, const Views &vs, cudaStream_t s) {
     ba.entries = c->entries.p;
     ba.entries_cap = (int64_t)c->entries.cap;
     ba.st = c->dstats.p;
-    launch_scatter(vs, ba, c->sms, s);
-    launch_fill_items(vs, c->offsets.p, c->item_offsets.p, c->items.p, (int)c->items.cap,
-                      c->dstats.p, seg_sms(c), s);
+    const ListArgs la{c->item_offsets.p, c->items.p, (int)c->items.cap, seg_sms(c), c->d_images.p, 0, 0, 0};
+    launch_lists(vs, ba, la, !c->accumulate, c->sms, s);
 }
 
 // Stage 3: schedule the work items, the tile and large passes, the epilogue.
@@ -816,7 +828,7 @@ static int render_views(spl_ctx *c, const spl_camera *cams, int V, float *const 
     SPL_CUDA(cudaGetLastError());
     const long long launched0 = g_launches;
     record_event(c, 0, s);
-    enqueue_binning(c, vs, s);
+    enqueue_binning(c, vs, false, s);
     SPL_CUDA(cudaGetLastError());
     SPL_CUDA(cudaMemcpyAsync(c->hstats, c->dstats.p, sizeof(DevStats), cudaMemcpyDeviceToHost, s));
     SPL_CUDA(cudaEventRecord(c->stats_ready, s));
@@ -1042,7 +1054,7 @@ static int capture_batch(spl_ctx *c, const Views &vs, unsigned long long key) {
     cudaError_t e = cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeRelaxed);
     if (e == cudaSuccess) {
         const long long launched0 = g_launches;
-        enqueue_binning(c, vs, c->cap_stream);
+        enqueue_binning(c, vs, true, c->cap_stream);
         enqueue_lists(c, vs, c->cap_stream);
         enqueue_passes(c, vs, true, c->cap_stream);
         c->graph_kernels = (int)(g_launches - launched0);
@@ -1377,7 +1389,7 @@ extern "C" int spl_count_work(spl_ctx *c, int64_t out[4]) {
     if (rc == SPL_OK) {
         const bool timing = c->timing;
         c->timing = false;
-        enqueue_binning(c, vs, s);
+        enqueue_binning(c, vs, false, s);
         c->timing = timing;
         launch_count_work(c->h_fcs[0], c->recs.p, c->n, work.p, c->sms, s);
         unsigned long long h[4] = {0, 0, 0, 0};
@@ -1421,7 +1433,9 @@ constexpr size_t kNaEntries = kNaCtab + na_round(sizeof(int2) * ctab_entries(kNa
 constexpr size_t kNaItems = kNaEntries + na_round(sizeof(unsigned) * kNaMaxEntries);
 constexpr size_t kNaView = kNaItems + na_round(sizeof(WorkItem) * kNaMaxItems);
 constexpr size_t kNaImage = kNaView + na_round(sizeof(FrameConst));
-constexpr size_t kNaBytes = kNaImage + na_round(sizeof(float *));
+constexpr size_t kNaPart = kNaImage + na_round(sizeof(float *));
+constexpr size_t kNaParts = 64;     // at least slot_parts(kNaMaxTiles)
+constexpr size_t kNaBytes = kNaPart + na_round(sizeof(long long) * kNaParts);
 }  // namespace
 
 static_assert(kNaBytes < ((size_t)17 << 20), "the fixed scratch stays below 17 MiB");
@@ -1511,6 +1525,8 @@ extern "C" int spl_render_noalloc(const spl_particles *p, const spl_camera *cam,
     WorkItem *items = reinterpret_cast<WorkItem *>(base + kNaItems);
     FrameConst *d_fc = reinterpret_cast<FrameConst *>(base + kNaView);
     float **d_img = reinterpret_cast<float **>(base + kNaImage);
+    long long *part = reinterpret_cast<long long *>(base + kNaPart);
+    if (slot_parts(fc.ntiles) > kNaParts) return SPL_ELIMIT;
     int sms = 1;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
     FrameConst fcv = fc;
@@ -1529,11 +1545,7 @@ extern "C" int spl_render_noalloc(const spl_particles *p, const spl_camera *cam,
     // (the error word stays: the previous call's passes may have set it, and
     // it is read at this call's synchronisation point)
     SPL_CUDA(cudaMemcpyAsync(pal, rgb, sizeof(float) * 3 * npal, cudaMemcpyHostToDevice, s));
-    SPL_CUDA(cudaMemcpyAsync(d_fc, &fcv, sizeof(FrameConst), cudaMemcpyHostToDevice, s));
-    SPL_CUDA(cudaMemcpyAsync(d_img, &d_image, sizeof(float *), cudaMemcpyHostToDevice, s));
-    SPL_CUDA(cudaMemsetAsync(dst, 0, offsetof(DevStats, err), s));
-    SPL_CUDA(cudaMemsetAsync(counts, 0, sizeof(int) * NLIST * fc.ntiles, s));
-    SPL_CUDA(cudaMemsetAsync(ovf, 0, sizeof(int) * NLIST * fc.ntiles, s));
+    launch_setup(SetupArgs{fcv, d_image, d_fc, d_img, counts, ovf, NLIST * fc.ntiles, dst}, sms, s);
     RasterArgs ra{};
     ra.n = p->n;
     ra.x = p->x; ra.y = p->y; ra.z = p->z;
@@ -1558,12 +1570,10 @@ extern "C" int spl_render_noalloc(const spl_particles *p, const spl_camera *cam,
     ba.cursor = cursor;
     ba.st = dst;
     launch_count_large(vs, ba, sms, s);
-    launch_slot_offsets(NLIST * fc.ntiles, counts, ovf, offsets, cursor, &dst->slot_total, s);
     // on images of up to 4096 tiles: the extra items (at most 8 per CTA of the passes
     // and list) then stay far below the fixed limit
     const int seg = fc.ntiles <= 4096 ? sms : 0;
-    launch_item_counts(vs, offsets, item_counts, dst, seg, s);
-    launch_scan(2 * fc.ntiles, item_counts, item_offsets, nullptr, 2, dst->item_totals, s);
+    launch_slots(vs, SlotArgs{counts, ovf, offsets, cursor, part, item_counts, item_offsets, dst}, seg, s);
     SPL_CUDA(cudaGetLastError());
     DevStats h;
     SPL_CUDA(cudaMemcpyAsync(&h, dst, sizeof(DevStats), cudaMemcpyDeviceToHost, s));
@@ -1577,11 +1587,9 @@ extern "C" int spl_render_noalloc(const spl_particles *p, const spl_camera *cam,
     const int n_tile_items = h.item_totals[0], n_large_items = h.item_totals[1];
     if (total > kNaMaxEntries || (int64_t)n_tile_items + n_large_items > kNaMaxItems)
         return SPL_ELIMIT;
-    launch_zero_images(vs, d_img, sms, s);
     ba.entries = entries;
     ba.entries_cap = kNaMaxEntries;
-    launch_scatter(vs, ba, sms, s);
-    launch_fill_items(vs, offsets, item_offsets, items, kNaMaxItems, dst, seg, s);
+    launch_lists(vs, ba, ListArgs{item_offsets, items, kNaMaxItems, seg, d_img, 0, 0, 0}, true, sms, s);
     TileArgs ta{};
     ta.recs = recs;
     ta.offsets = offsets;

@@ -193,23 +193,45 @@ constexpr int kNParam = kHid * kFeat + 2 * kHid + 1;
 // the whole sequence can be captured in a CUDA graph.
 void launch_raster(const Views &v, const RasterArgs &a, int attr, cudaStream_t s);
 void launch_count_large(const Views &v, const BinArgs &a, int sms, cudaStream_t s);
-// Slot offsets and cursors from counts + ovf (ovf is overwritten with the sums).
-void launch_slot_offsets(int m, int *counts, int *ovf, long long *offsets, long long *cursor,
-                         long long *total, cudaStream_t s);
 
-// Exclusive scan of in[0..m) into out[0..m] (out[m] = total); cursor (may be
-// null) receives a copy of out[0..m); seg_totals[k] = total of the k-th of
-// nseg equal segments.
-void launch_scan(int m, const int *in, long long *out, long long *cursor, int nseg,
-                 long long *seg_totals, cudaStream_t s);
-void launch_scan(int m, const int *in, int *out, int *cursor, int nseg, int *seg_totals,
-                 cudaStream_t s);
-// sms > 0: segments shrink on small frames (see kSegShrink); 0: full segments.
-void launch_item_counts(const Views &v, const long long *offsets, int *item_counts, DevStats *st,
-                        int sms, cudaStream_t s);
-void launch_fill_items(const Views &v, const long long *offsets, const int *item_offsets,
-                       WorkItem *items, int items_cap, DevStats *st, int sms, cudaStream_t s);
-void launch_scatter(const Views &v, const BinArgs &a, int sms, cudaStream_t s);
+// The start of a frame: zeroes the slot counts and the frame's statistics; a single
+// view's constants and image (fcs not null) are written from the arguments.
+struct SetupArgs {
+    FrameConst fc;
+    float *image;
+    FrameConst *fcs;           // device, or null: copied by the caller
+    float **images;
+    int *counts, *ovf;
+    int slots;
+    DevStats *st;
+};
+void launch_setup(const SetupArgs &a, int sms, cudaStream_t s);
+
+// Slot counts and ovf to list offsets, cursors, item offsets ([tile-pass items | large
+// items]) and the totals in st.  sms > 0: segments shrink on small frames (see
+// kSegShrink); 0: full segments.  part: slot_parts(total_tiles) values of scratch.
+struct SlotArgs {
+    const int *counts, *ovf;
+    long long *offsets, *cursor, *part;
+    int *item_counts, *item_offsets;
+    DevStats *st;
+};
+void launch_slots(const Views &v, const SlotArgs &a, int sms, cudaStream_t s);
+size_t slot_parts(int tiles);
+
+// Exclusive scan of in[0..m) into out[0..m] (out[m] = total).
+void launch_scan(int m, const int *in, int *out, cudaStream_t s);
+
+// The tile lists, the work items and (zero) the cleared images.  The caller fills the
+// first five fields of l.
+struct ListArgs {
+    const int *item_offsets;
+    WorkItem *items;
+    int items_cap, seg_sms;
+    float *const *images;
+    int large_blocks, item_blocks, zero_blocks;
+};
+void launch_lists(const Views &v, const BinArgs &a, ListArgs l, bool zero, int sms, cudaStream_t s);
 void launch_tile_pass(const Views &v, const TileArgs &a, int sms, cudaStream_t s);
 void launch_large_pass(const Views &v, const TileArgs &a, int sms, cudaStream_t s);
 // Absorption mode: the depth-ordered pass and the composition of split tiles.
@@ -229,9 +251,8 @@ void launch_encode_attrs(const float *h, const float *I, const float *s, int64_t
 // cursor[k] = offsets[k] + counts[k] for the m list slots (re-arms the scatter).
 void launch_slot_cursor(int m, const int *counts, const long long *offsets, long long *cursor,
                         cudaStream_t s);
-// Zero every view's image / apply the E=A map to every view's image (the
-// image pointers are read from device memory, so a graph can replay them).
-void launch_zero_images(const Views &v, float *const *images, int sms, cudaStream_t s);
+// Apply the E=A map to every view's image (the image pointers are read from
+// device memory, so a graph can replay them).
 void launch_epilogue_views(const Views &v, float *const *images, int sms, cudaStream_t s);
 void launch_count_work(const FrameConst &fc, const Rec *recs, int64_t n,
                        unsigned long long *work, int sms, cudaStream_t s);

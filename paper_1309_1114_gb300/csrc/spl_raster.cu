@@ -2,6 +2,8 @@
 // Sec. 4 one-thread-per-particle) and binning of particles into tile lists
 // (the data organisation of Sec. 4, built with counts, a scan and a scatter
 // instead of a radix sort by tile index).
+#include <cstddef>
+
 #include "spl_geom.cuh"
 
 namespace spl {
@@ -444,11 +446,12 @@ void launch_raster(const Views &vs, const RasterArgs &a, int attr, cudaStream_t 
 // the cursors.
 // ---------------------------------------------------------------------------
 template <int MODE>
-__global__ void __launch_bounds__(256) large_tiles_kernel(Views vs, BinArgs a) {
+__device__ __forceinline__ void large_tiles(const Views &vs, const BinArgs &a, unsigned block,
+                                            unsigned nblocks) {
     const int lane = threadIdx.x & 31;
     const unsigned nl = a.st->n_large_ids;
-    const unsigned warps = gridDim.x * (blockDim.x >> 5);
-    for (unsigned w = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); w < nl; w += warps) {
+    const unsigned warps = nblocks * (blockDim.x >> 5);
+    for (unsigned w = block * (blockDim.x >> 5) + (threadIdx.x >> 5); w < nl; w += warps) {
         const unsigned rec = a.large_ids[w];
         const FrameConst &fc = vs.fcs[(int)(rec / (unsigned long long)vs.n)];
         const Rec rc = a.recs[rec];
@@ -477,15 +480,14 @@ __global__ void __launch_bounds__(256) large_tiles_kernel(Views vs, BinArgs a) {
     }
 }
 
-void launch_count_large(const Views &vs, const BinArgs &a, int sms, cudaStream_t s) {
-    if (vs.n <= 0) return;
-    large_tiles_kernel<0><<<sms * 2, 256, 0, s>>>(vs, a);
-    ++g_launches;
+__global__ void __launch_bounds__(256) count_large_kernel(Views vs, BinArgs a) {
+    large_tiles<0>(vs, a, blockIdx.x, gridDim.x);
 }
 
-__global__ void slot_sum_kernel(int m, const int *counts, int *ovf) {
-    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < m; k += gridDim.x * blockDim.x)
-        ovf[k] += counts[k];
+void launch_count_large(const Views &vs, const BinArgs &a, int sms, cudaStream_t s) {
+    if (vs.n <= 0) return;
+    count_large_kernel<<<sms * 2, 256, 0, s>>>(vs, a);
+    ++g_launches;
 }
 
 __global__ void slot_cursor_kernel(int m, const int *counts, const long long *offsets,
@@ -494,60 +496,56 @@ __global__ void slot_cursor_kernel(int m, const int *counts, const long long *of
         cursor[k] = offsets[k] + counts[k];
 }
 
-// ---------------------------------------------------------------------------
-// Exclusive scan: one CTA of 1024 threads, each owning a contiguous run.
-// ---------------------------------------------------------------------------
-template <typename OT>
-__global__ void __launch_bounds__(1024) scan_kernel(int m, const int *in, OT *out, OT *cursor,
-                                                    int nseg, OT *seg_totals) {
-    __shared__ OT wsum[32];
-    const int t = threadIdx.x, per = (m + 1023) / 1024;
-    const int lo = min(t * per, m), hi = min(lo + per, m);
-    OT sum = 0;
-    for (int k = lo; k < hi; ++k) sum += (OT)in[k];
-    const int lane = t & 31, warp = t >> 5;
-    OT incl = sum;
+// Exclusive scan of one value per thread over a block of 1024 threads (wsum: 33).
+template <typename V>
+__device__ __forceinline__ V block_scan(V v, V *wsum, V &total) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    V incl = v;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
-        OT v = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += v;
+        const V u = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += u;
     }
     if (lane == 31) wsum[warp] = incl;
     __syncthreads();
     if (warp == 0) {
-        OT v = wsum[lane];
-        OT w = v;
+        const V w = wsum[lane];
+        V wi = w;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
-            OT u = __shfl_up_sync(0xffffffffu, w, o);
-            if (lane >= o) w += u;
+            const V u = __shfl_up_sync(0xffffffffu, wi, o);
+            if (lane >= o) wi += u;
         }
-        wsum[lane] = w - v;
+        wsum[lane] = wi - w;
+        if (lane == 31) wsum[32] = wi;
     }
     __syncthreads();
-    OT run = wsum[warp] + incl - sum;
+    total = wsum[32];
+    const V r = wsum[warp] + incl - v;
+    __syncthreads();
+    return r;
+}
+
+// ---------------------------------------------------------------------------
+// Exclusive scan: one CTA of 1024 threads, each owning a contiguous run.
+// ---------------------------------------------------------------------------
+__global__ void __launch_bounds__(1024) scan_kernel(int m, const int *in, int *out) {
+    __shared__ int wsum[33];
+    const int t = threadIdx.x, per = (m + 1023) / 1024;
+    const int lo = min(t * per, m), hi = min(lo + per, m);
+    int sum = 0;
+    for (int k = lo; k < hi; ++k) sum += in[k];
+    int total;
+    int run = block_scan(sum, wsum, total);
     for (int k = lo; k < hi; ++k) {
         out[k] = run;
-        if (cursor) cursor[k] = run;
-        run += (OT)in[k];
+        run += in[k];
     }
-    if (t == 1023) out[m] = run;
-    __syncthreads();   // makes every thread's results visible to the block
-    if (t < nseg) {
-        const int seg = m / nseg;
-        seg_totals[t] = out[(t + 1) * seg] - out[t * seg];
-    }
+    if (t == 0) out[m] = total;
 }
 
-void launch_scan(int m, const int *in, long long *out, long long *cursor, int nseg,
-                 long long *seg_totals, cudaStream_t s) {
-    scan_kernel<long long><<<1, 1024, 0, s>>>(m, in, out, cursor, nseg, seg_totals);
-    ++g_launches;
-}
-
-void launch_scan(int m, const int *in, int *out, int *cursor, int nseg, int *seg_totals,
-                 cudaStream_t s) {
-    scan_kernel<int><<<1, 1024, 0, s>>>(m, in, out, cursor, nseg, seg_totals);
+void launch_scan(int m, const int *in, int *out, cudaStream_t s) {
+    scan_kernel<<<1, 1024, 0, s>>>(m, in, out);
     ++g_launches;
 }
 
@@ -559,21 +557,6 @@ void launch_slot_cursor(int m, const int *counts, const long long *offsets, long
     ++g_launches;
 }
 
-void launch_slot_offsets(int m, int *counts, int *ovf, long long *offsets, long long *cursor,
-                         long long *total, cudaStream_t s) {
-    const int grid = (m + 255) / 256 < 1024 ? (m + 255) / 256 : 1024;
-    if (grid > 0) {
-        slot_sum_kernel<<<grid, 256, 0, s>>>(m, counts, ovf);
-        ++g_launches;
-    }
-    scan_kernel<long long><<<1, 1024, 0, s>>>(m, ovf, offsets, nullptr, 1, total);
-    ++g_launches;
-    if (grid > 0) {
-        slot_cursor_kernel<<<grid, 256, 0, s>>>(m, counts, offsets, cursor);
-        ++g_launches;
-    }
-}
-
 // ---------------------------------------------------------------------------
 // Work items: a light tile is one item (all its lists, pixels stored); a
 // crowded tile is cut into segments of at most kSeg* entries per list (fewer on
@@ -582,79 +565,225 @@ void launch_slot_offsets(int m, int *counts, int *ovf, long long *offsets, long 
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ int div_up(int a, int b) { return (a + b - 1) / b; }
 
-// Segment lengths of this frame, the same in every CTA that asks (the lists' totals
-// are differences of their first and last offsets, summed over the views).  The
-// weights are the lists' cost per entry in the tile pass, in medium entries.
-__device__ __forceinline__ void frame_segs(const Views &vs, const long long *off, int sms, Segs *segs,
-                                           unsigned long long *tot) {
+// Entries per list of this frame, summed over the views (differences of the lists'
+// first and last offsets), into tot[NLIST]; the whole block takes part.
+__device__ __forceinline__ void list_totals(const Views &vs, const long long *off,
+                                            unsigned long long *tot) {
     if (threadIdx.x < NLIST) tot[threadIdx.x] = 0ull;
     __syncthreads();
-    if (sms > 0)
-        for (int k = threadIdx.x; k < vs.nviews * NLIST; k += blockDim.x) {
-            const FrameConst &fc = vs.fcs[k / NLIST];
-            const int l = k % NLIST, b = fc.slot_base + l * fc.ntiles;
-            atomicAdd(&tot[l], (unsigned long long)(off[b + fc.ntiles] - off[b]));
-        }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        const int full[NLIST] = {kSegPoint, kSegSmall, kSegMedium, kSegLarge};
-        // CTAs of the passes: 4 per SM; two segments each
-        const unsigned long long work = tot[L_MEDIUM] + tot[L_SMALL] / 8 + tot[L_POINT] / 64;
-        for (int l = 0; l < NLIST; ++l) {
-            const int whole = l == L_LARGE ? kSegLarge : kSegMedium;
-            long long len = whole;
-            if (sms > 0) {
-                len = (long long)((l == L_LARGE ? tot[L_LARGE] : work) / (unsigned long long)(8 * sms));
-                len = (len + 63) / 64 * 64;
-                len = len < whole / kSegShrink ? whole / kSegShrink : (len > whole ? whole : len);
-            }
-            segs->len[l] = (int)(full[l] / whole * len);
-        }
+    for (int k = threadIdx.x; k < vs.nviews * NLIST; k += blockDim.x) {
+        const FrameConst &fc = vs.fcs[k / NLIST];
+        const int b = fc.slot_base + k % NLIST * fc.ntiles;
+        atomicAdd(&tot[k % NLIST], (unsigned long long)(off[b + fc.ntiles] - off[b]));
     }
     __syncthreads();
 }
 
-__global__ void item_count_kernel(Views vs, const long long *off, int *item_counts, DevStats *st,
-                                  int sms) {
-    __shared__ int lt[NLIST];
-    __shared__ Segs segs;
-    __shared__ unsigned long long tots[NLIST];
-    if (threadIdx.x < NLIST) lt[threadIdx.x] = 0;
-    frame_segs(vs, off, sms, &segs, tots);
-    const int T = vs.total_tiles;
-    int tot[NLIST] = {0, 0, 0, 0};
-    for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < T; g += gridDim.x * blockDim.x) {
-        const FrameConst &fc = vs.fcs[view_of_tile(vs.fcs, vs.nviews, g)];
-        const int t = g - fc.tile_base, nt = fc.ntiles, sb = fc.slot_base;
-        const int cp = (int)(off[sb + L_POINT * nt + t + 1] - off[sb + L_POINT * nt + t]);
-        const int cs = (int)(off[sb + L_SMALL * nt + t + 1] - off[sb + L_SMALL * nt + t]);
-        const int cm = (int)(off[sb + L_MEDIUM * nt + t + 1] - off[sb + L_MEDIUM * nt + t]);
-        const int cl = (int)(off[sb + L_LARGE * nt + t + 1] - off[sb + L_LARGE * nt + t]);
-        tot[0] += cp; tot[1] += cs; tot[2] += cm; tot[3] += cl;
-        int n = 0;
-        if (cp + cs + cm > 0) {
-            if (cp <= segs.len[L_POINT] && cs <= segs.len[L_SMALL] && cm <= segs.len[L_MEDIUM])
-                n = 1;
-            else
-                n = div_up(cp, segs.len[L_POINT]) + div_up(cs, segs.len[L_SMALL]) +
-                    div_up(cm, segs.len[L_MEDIUM]);
-        }
-        item_counts[g] = n;
-        item_counts[T + g] = div_up(cl, segs.len[L_LARGE]);
-    }
+// Segment lengths of a frame with these totals (see kSegShrink).  The weights are the
+// lists' cost per entry in the tile pass, in medium entries.
+__device__ __forceinline__ Segs frame_segs(const unsigned long long *tot, int sms) {
+    const int full[NLIST] = {kSegPoint, kSegSmall, kSegMedium, kSegLarge};
+    // CTAs of the passes: 4 per SM; two segments each
+    const unsigned long long work = tot[L_MEDIUM] + tot[L_SMALL] / 8 + tot[L_POINT] / 64;
+    Segs segs;
+#pragma unroll
     for (int l = 0; l < NLIST; ++l) {
-        const int v = __reduce_add_sync(0xffffffffu, tot[l]);
-        if ((threadIdx.x & 31) == 0 && v) atomicAdd(&lt[l], v);
+        const int whole = l == L_LARGE ? kSegLarge : kSegMedium;
+        long long len = whole;
+        if (sms > 0) {
+            len = (long long)((l == L_LARGE ? tot[L_LARGE] : work) / (unsigned long long)(8 * sms));
+            len = (len + 63) / 64 * 64;
+            len = len < whole / kSegShrink ? whole / kSegShrink : (len > whole ? whole : len);
+        }
+        segs.len[l] = (int)(full[l] / whole * len);
     }
-    __syncthreads();
-    if (threadIdx.x < NLIST && lt[threadIdx.x]) atomicAdd(&st->totals[threadIdx.x], lt[threadIdx.x]);
+    return segs;
 }
 
-void launch_item_counts(const Views &vs, const long long *offsets, int *item_counts, DevStats *st,
-                        int sms, cudaStream_t s) {
-    const int blocks = (vs.total_tiles + 255) / 256;
-    item_count_kernel<<<blocks, 256, 0, s>>>(vs, offsets, item_counts, st, sms);
-    ++g_launches;
+// Items of global tile g: of the tile pass, and of the large pass in *large.
+__device__ __forceinline__ int tile_items(const Views &vs, const long long *off, const Segs &segs, int g,
+                                          int *large) {
+    const FrameConst &fc = vs.fcs[view_of_tile(vs.fcs, vs.nviews, g)];
+    const int nt = fc.ntiles;
+    const long long *o = off + fc.slot_base + g - fc.tile_base;
+    const int cp = (int)(o[L_POINT * nt + 1] - o[L_POINT * nt]);
+    const int cs = (int)(o[L_SMALL * nt + 1] - o[L_SMALL * nt]);
+    const int cm = (int)(o[L_MEDIUM * nt + 1] - o[L_MEDIUM * nt]);
+    const int cl = (int)(o[L_LARGE * nt + 1] - o[L_LARGE * nt]);
+    *large = div_up(cl, segs.len[L_LARGE]);
+    if (cp + cs + cm == 0) return 0;
+    if (cp <= segs.len[L_POINT] && cs <= segs.len[L_SMALL] && cm <= segs.len[L_MEDIUM]) return 1;
+    return div_up(cp, segs.len[L_POINT]) + div_up(cs, segs.len[L_SMALL]) + div_up(cm, segs.len[L_MEDIUM]);
+}
+
+// ---------------------------------------------------------------------------
+// From the slot counts to the list offsets and the item offsets.  Frames of up to
+// kSlotChunk slots (1024 tiles) take one CTA and one launch; larger ones four
+// launches of one chunk per CTA, each CTA adding up the chunks before its own.
+// One CTA walking contiguous runs per thread, and a launch for each of the sum, scan,
+// cursor, item count and item scan, took 10 us on a small frame and 170 us at 16384
+// tiles (now 4 and 12 us).
+// ---------------------------------------------------------------------------
+constexpr int kSlotChunk = 4096, kItemChunk = 1024;
+
+// This thread's four slots of a chunk: offsets and cursors from base.
+__device__ __forceinline__ void put_slots(int k, int m, const int *c, const int *o, long long run,
+                                          long long *offsets, long long *cursor) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+        if (k + q < m) {
+            offsets[k + q] = run;
+            cursor[k + q] = run + c[q];
+            run += c[q] + o[q];
+        }
+}
+
+__device__ __forceinline__ long long get_slots(int k, int m, const int *counts, const int *ovf, int *c,
+                                               int *o) {
+    long long sum = 0;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        c[q] = k + q < m ? counts[k + q] : 0;
+        o[q] = k + q < m ? ovf[k + q] : 0;
+        sum += c[q] + o[q];
+    }
+    return sum;
+}
+
+__global__ void __launch_bounds__(1024) slots_kernel(Views vs, int m, const int *counts, const int *ovf,
+                                                     long long *offsets, long long *cursor, int *ioff,
+                                                     DevStats *st, int sms) {
+    __shared__ long long wsum[33];
+    __shared__ int isum[33];
+    __shared__ unsigned long long tot[NLIST];
+    const int t = threadIdx.x;
+    int c[4], o[4];
+    long long total;
+    const long long run = block_scan(get_slots(4 * t, m, counts, ovf, c, o), wsum, total);
+    put_slots(4 * t, m, c, o, run, offsets, cursor);
+    if (t == 0) {
+        offsets[m] = total;
+        st->slot_total = total;
+    }
+    __syncthreads();                       // the block's own offsets are visible to it
+    list_totals(vs, offsets, tot);
+    if (t < NLIST) st->totals[t] = (int)tot[t];
+    const Segs segs = frame_segs(tot, sms);
+    const int T = vs.total_tiles;
+    int large = 0;
+    const int n = t < T ? tile_items(vs, offsets, segs, t, &large) : 0;
+    int n_tile, n_large;
+    const int at = block_scan(n, isum, n_tile), lat = block_scan(large, isum, n_large);
+    if (t < T) {
+        ioff[t] = at;
+        ioff[T + t] = n_tile + lat;
+    }
+    if (t == 0) {
+        ioff[2 * T] = n_tile + n_large;
+        st->item_totals[0] = n_tile;
+        st->item_totals[1] = n_large;
+    }
+}
+
+__global__ void __launch_bounds__(1024) slot_reduce_kernel(int m, const int *counts, const int *ovf,
+                                                           long long *part) {
+    __shared__ long long wsum[33];
+    int c[4], o[4];
+    long long total;
+    block_scan(get_slots(blockIdx.x * kSlotChunk + 4 * threadIdx.x, m, counts, ovf, c, o), wsum, total);
+    if (threadIdx.x == 0) part[blockIdx.x] = total;
+}
+
+__global__ void __launch_bounds__(1024) slot_apply_kernel(int m, const int *counts, const int *ovf,
+                                                          const long long *part, long long *offsets,
+                                                          long long *cursor, DevStats *st) {
+    __shared__ long long wsum[33];
+    const int k = blockIdx.x * kSlotChunk + 4 * threadIdx.x;
+    long long before = 0, base, total;
+    for (int b = threadIdx.x; b < (int)blockIdx.x; b += 1024) before += part[b];
+    block_scan(before, wsum, base);
+    int c[4], o[4];
+    const long long sum = get_slots(k, m, counts, ovf, c, o);
+    const long long run = base + block_scan(sum, wsum, total);
+    put_slots(k, m, c, o, run, offsets, cursor);
+    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) {
+        offsets[m] = base + total;
+        st->slot_total = base + total;
+    }
+}
+
+__global__ void __launch_bounds__(kItemChunk) item_count_kernel(Views vs, const long long *off,
+                                                                int *item_counts, int *part,
+                                                                DevStats *st, int sms) {
+    __shared__ unsigned long long tot[NLIST];
+    __shared__ int isum[33];
+    list_totals(vs, off, tot);
+    if (blockIdx.x == 0 && threadIdx.x < NLIST) st->totals[threadIdx.x] = (int)tot[threadIdx.x];
+    const Segs segs = frame_segs(tot, sms);
+    const int T = vs.total_tiles, g = blockIdx.x * kItemChunk + threadIdx.x;
+    int large = 0, n = 0, n_tile, n_large;
+    if (g < T) {
+        n = tile_items(vs, off, segs, g, &large);
+        item_counts[g] = n;
+        item_counts[T + g] = large;
+    }
+    block_scan(n, isum, n_tile);
+    block_scan(large, isum, n_large);
+    if (threadIdx.x == 0) {
+        part[blockIdx.x] = n_tile;
+        part[gridDim.x + blockIdx.x] = n_large;
+    }
+}
+
+__global__ void __launch_bounds__(kItemChunk) item_apply_kernel(int T, const int *item_counts,
+                                                                const int *part, int *ioff,
+                                                                DevStats *st) {
+    __shared__ int isum[33];
+    const int nb = gridDim.x, g = blockIdx.x * kItemChunk + threadIdx.x;
+    int tb = 0, ta = 0, lb = 0;            // tile items before, tile items of all, large items before
+    for (int b = threadIdx.x; b < nb; b += kItemChunk) {
+        ta += part[b];
+        if (b < (int)blockIdx.x) {
+            tb += part[b];
+            lb += part[nb + b];
+        }
+    }
+    int tile_before, tile_all, large_before, n_tile, n_large;
+    block_scan(tb, isum, tile_before);
+    block_scan(ta, isum, tile_all);
+    block_scan(lb, isum, large_before);
+    const int at = block_scan(g < T ? item_counts[g] : 0, isum, n_tile);
+    const int lat = block_scan(g < T ? item_counts[T + g] : 0, isum, n_large);
+    if (g < T) {
+        ioff[g] = tile_before + at;
+        ioff[T + g] = tile_all + large_before + lat;
+    }
+    if ((int)blockIdx.x == nb - 1 && threadIdx.x == 0) {
+        ioff[2 * T] = tile_all + large_before + n_large;
+        st->item_totals[0] = tile_all;
+        st->item_totals[1] = large_before + n_large;
+    }
+}
+
+void launch_slots(const Views &vs, const SlotArgs &a, int sms, cudaStream_t s) {
+    const int T = vs.total_tiles, m = NLIST * T;
+    if (m <= kSlotChunk) {
+        slots_kernel<<<1, 1024, 0, s>>>(vs, m, a.counts, a.ovf, a.offsets, a.cursor, a.item_offsets, a.st,
+                                        sms);
+        ++g_launches;
+        return;
+    }
+    const int nb = (m + kSlotChunk - 1) / kSlotChunk, ni = (T + kItemChunk - 1) / kItemChunk;
+    int *ipart = reinterpret_cast<int *>(a.part + nb);
+    slot_reduce_kernel<<<nb, 1024, 0, s>>>(m, a.counts, a.ovf, a.part);
+    slot_apply_kernel<<<nb, 1024, 0, s>>>(m, a.counts, a.ovf, a.part, a.offsets, a.cursor, a.st);
+    item_count_kernel<<<ni, kItemChunk, 0, s>>>(vs, a.offsets, a.item_counts, ipart, a.st, sms);
+    item_apply_kernel<<<ni, kItemChunk, 0, s>>>(T, a.item_counts, ipart, a.item_offsets, a.st);
+    g_launches += 4;
+}
+
+size_t slot_parts(int tiles) {
+    return (size_t)(NLIST * (int64_t)tiles / kSlotChunk + 1) + (size_t)tiles / kItemChunk + 1;
 }
 
 __device__ __forceinline__ void put_item(WorkItem *items, int cap, int pos, WorkItem w, DevStats *st) {
@@ -666,16 +795,17 @@ __device__ __forceinline__ void put_item(WorkItem *items, int cap, int pos, Work
 
 // One warp per tile: the lanes write the tile's segments side by side (a
 // crowded tile has hundreds), in the same order as one thread would.
-__global__ void fill_items_kernel(Views vs, const long long *off, const int *ioff, WorkItem *items,
-                                  int cap, DevStats *st, int sms) {
+__device__ __forceinline__ void fill_items(const Views &vs, const long long *off, const int *ioff,
+                                           WorkItem *items, int cap, DevStats *st, int sms, int block,
+                                           int nblocks) {
     const int T = vs.total_tiles;
-    __shared__ Segs segs;
-    __shared__ unsigned long long tots[NLIST];
-    frame_segs(vs, off, sms, &segs, tots);
+    __shared__ unsigned long long tot[NLIST];
+    list_totals(vs, off, tot);
+    const Segs segs = frame_segs(tot, sms);
     const int *seg = segs.len;
     const int lane = threadIdx.x & 31;
-    const int warps = (gridDim.x * blockDim.x) >> 5;
-    for (int g = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; g < T; g += warps) {
+    const int warps = (nblocks * blockDim.x) >> 5;
+    for (int g = (block * blockDim.x + threadIdx.x) >> 5; g < T; g += warps) {
         const int v = view_of_tile(vs.fcs, vs.nviews, g);
         const FrameConst &fc = vs.fcs[v];
         const int t = g - fc.tile_base, nt = fc.ntiles, sb = fc.slot_base;
@@ -708,13 +838,6 @@ __global__ void fill_items_kernel(Views vs, const long long *off, const int *iof
     }
 }
 
-void launch_fill_items(const Views &vs, const long long *offsets, const int *item_offsets,
-                       WorkItem *items, int items_cap, DevStats *st, int sms, cudaStream_t s) {
-    const int blocks = (vs.total_tiles + 7) / 8;     // 8 warps of 256 threads, a warp per tile
-    fill_items_kernel<<<blocks, 256, 0, s>>>(vs, offsets, item_offsets, items, items_cap, st, sms);
-    ++g_launches;
-}
-
 // ---------------------------------------------------------------------------
 // Scatter particle ids of points, small and medium particles into their
 // tiles' lists (order inside a tile follows the atomics, which is harmless:
@@ -741,20 +864,20 @@ __device__ __forceinline__ TileFoot load_foot(const FrameConst &fc, const BinArg
 // Keys that had no room in the table go through the cursors.  Order inside a
 // tile follows the atomics, which is harmless: E_p = A_p makes the sum
 // order-independent (Sec. 2); the absorption mode sorts the lists afterwards.
-__global__ void __launch_bounds__(256) scatter_kernel(Views vs, BinArgs a) {
-    extern __shared__ long long scatter_smem[];
+__device__ __forceinline__ void scatter_chunk(const Views &vs, const BinArgs &a, int block,
+                                              long long *scatter_smem) {
     long long *bases = scatter_smem;                         // kHash
     int *keys = reinterpret_cast<int *>(bases + kHash);      // kHash
     int *vals = keys + kHash;                                // kHash
     __shared__ FrameConst sfc;
     const int lane = threadIdx.x & 31;
     const unsigned lt = (1u << lane) - 1u;
-    const int64_t c0 = (int64_t)blockIdx.x * kChunk;
+    const int64_t c0 = (int64_t)block * kChunk;
     const int64_t c1 = c0 + kChunk < vs.n ? c0 + kChunk : vs.n;
     for (int v = 0; v < vs.nviews; ++v) {
         load_view(vs.fcs, v, &sfc);     // (begins and ends with a barrier)
         const FrameConst &fc = sfc;
-        const int2 *tab = a.ctab + ((int64_t)blockIdx.x * vs.nviews + v) * kHash;
+        const int2 *tab = a.ctab + ((int64_t)block * vs.nviews + v) * kHash;
         for (int k = threadIdx.x; k < kHash; k += blockDim.x) {
             const int2 t = tab[k];
             keys[k] = t.x;
@@ -797,14 +920,70 @@ __global__ void __launch_bounds__(256) scatter_kernel(Views vs, BinArgs a) {
     }
 }
 
-void launch_scatter(const Views &vs, const BinArgs &a, int sms, cudaStream_t s) {
-    if (vs.n <= 0 || vs.nviews <= 0) return;
-    const int64_t blocks = (vs.n + kChunk - 1) / kChunk;
+// Everything that follows the offsets, in one launch, by the block's number: the large
+// lists, the work items and the cleared images are a few blocks' work beside the
+// scatter, and each was a launch of its own.
+__global__ void __launch_bounds__(256, 6) lists_kernel(Views vs, BinArgs a, ListArgs l) {
+    extern __shared__ long long lists_smem[];
+    int b = blockIdx.x;
+    if (b < l.large_blocks) {
+        large_tiles<1>(vs, a, b, l.large_blocks);
+        return;
+    }
+    b -= l.large_blocks;
+    if (b < l.item_blocks) {
+        fill_items(vs, a.offsets, l.item_offsets, l.items, l.items_cap, a.st, l.seg_sms, b, l.item_blocks);
+        return;
+    }
+    b -= l.item_blocks;
+    if (b < l.zero_blocks) {
+        for (int v = 0; v < vs.nviews; ++v) {
+            const int64_t n = (int64_t)3 * vs.fcs[v].width * vs.fcs[v].height;
+            float *img = l.images[v];
+            for (int64_t i = (int64_t)b * blockDim.x + threadIdx.x; i < n;
+                 i += (int64_t)l.zero_blocks * blockDim.x)
+                img[i] = 0.f;
+        }
+        return;
+    }
+    scatter_chunk(vs, a, b - l.zero_blocks, lists_smem);
+}
+
+void launch_lists(const Views &vs, const BinArgs &a, ListArgs l, bool zero, int sms, cudaStream_t s) {
+    const int64_t chunks = vs.n > 0 ? (vs.n + kChunk - 1) / kChunk : 0;
     const size_t smem = (size_t)kHash * (sizeof(long long) + 2 * sizeof(int));
-    cudaFuncSetAttribute(scatter_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    scatter_kernel<<<(unsigned)blocks, 256, smem, s>>>(vs, a);
+    l.large_blocks = vs.n > 0 ? sms * 2 : 0;
+    const int warps = (vs.total_tiles + 7) / 8;     // 8 warps of 256 threads, a warp per tile
+    l.item_blocks = warps < sms * 4 ? warps : sms * 4;
+    l.zero_blocks = zero ? sms * 2 : 0;
+    cudaFuncSetAttribute(lists_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const int64_t blocks = l.large_blocks + l.item_blocks + l.zero_blocks + chunks;
+    lists_kernel<<<(unsigned)blocks, 256, smem, s>>>(vs, a, l);
     ++g_launches;
-    large_tiles_kernel<1><<<sms * 2, 256, 0, s>>>(vs, a);
+}
+
+// ---------------------------------------------------------------------------
+// The start of a frame: the view's constants (a single view's travel as launch
+// arguments) and everything that starts at zero.  Three memsets and two copies took
+// as many slots of the stream.
+// ---------------------------------------------------------------------------
+__global__ void __launch_bounds__(256) setup_kernel(const __grid_constant__ SetupArgs a) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x, stride = gridDim.x * blockDim.x;
+    for (int k = i; k < a.slots; k += stride) {
+        a.counts[k] = 0;
+        a.ovf[k] = 0;
+    }
+    if (i < (int)(offsetof(DevStats, err) / sizeof(int))) reinterpret_cast<int *>(a.st)[i] = 0;
+    if (a.fcs) {
+        if (i < (int)(sizeof(FrameConst) / sizeof(int)))
+            reinterpret_cast<int *>(a.fcs)[i] = reinterpret_cast<const int *>(&a.fc)[i];
+        if (i == 0) *a.images = a.image;
+    }
+}
+
+void launch_setup(const SetupArgs &a, int sms, cudaStream_t s) {
+    const int blocks = (a.slots + 255) / 256;
+    setup_kernel<<<blocks < 1 ? 1 : (blocks < sms * 4 ? blocks : sms * 4), 256, 0, s>>>(a);
     ++g_launches;
 }
 

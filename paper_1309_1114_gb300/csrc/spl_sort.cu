@@ -185,7 +185,7 @@ static void scan_digits(int m, const int *in, int *out, int *part, int *pbase, c
     const int np = scan_parts(m);
     scan_reduce_kernel<<<np, kScanThreads, 0, s>>>(in, m, part);
     ++g_launches;
-    launch_scan(np, part, pbase, nullptr, 0, nullptr, s);
+    launch_scan(np, part, pbase, s);
     scan_apply_kernel<<<np, kScanThreads, 0, s>>>(in, m, pbase, np, out);
     ++g_launches;
 }

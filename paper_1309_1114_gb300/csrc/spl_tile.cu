@@ -811,24 +811,18 @@ void launch_epilogue_ea(float *image, int64_t nvals, int sms, cudaStream_t s) {
 }
 
 // Grid-stride over every pixel value of every view (blockIdx.y = view).
-template <bool EA>
-__global__ void views_pointwise_kernel(Views vs, float *const *images) {
+__global__ void views_ea_kernel(Views vs, float *const *images) {
     const int v = blockIdx.y;
     const FrameConst &fc = vs.fcs[v];
     float *img = images[v];
     const int64_t n = (int64_t)3 * fc.width * fc.height;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride)
-        img[i] = EA ? -expm1f(-img[i]) : 0.f;
-}
-
-void launch_zero_images(const Views &vs, float *const *images, int sms, cudaStream_t s) {
-    views_pointwise_kernel<false><<<dim3(sms * 2, vs.nviews), 256, 0, s>>>(vs, images);
-    ++g_launches;
+        img[i] = -expm1f(-img[i]);
 }
 
 void launch_epilogue_views(const Views &vs, float *const *images, int sms, cudaStream_t s) {
-    views_pointwise_kernel<true><<<dim3(sms * 2, vs.nviews), 256, 0, s>>>(vs, images);
+    views_ea_kernel<<<dim3(sms * 2, vs.nviews), 256, 0, s>>>(vs, images);
     ++g_launches;
 }
 
