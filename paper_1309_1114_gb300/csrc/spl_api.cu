@@ -774,7 +774,10 @@ static void enqueue_passes(spl_ctx *c, const Views &vs, bool large_pass, cudaStr
         launch_order_items(c->cost.p, ta.items_cap, c->dstats.p, c->order_hist.p, c->order.p, s);
         ta.order = c->order.p;
     }
-    if (c->recording) ta.item_cycles = c->item_cycles.p;
+    if (c->recording) {
+        ta.item_cycles = c->item_cycles.p;
+        cudaMemsetAsync(ta.item_cycles, 0, sizeof(long long) * c->item_cycles.cap, s);
+    }
     if (c->par.mode == SPL_MODE_ABSORB) {
         // one view: every entry sits in the medium slots [L_MEDIUM * nt, (L_MEDIUM + 1) * nt]
         const int nt = c->h_fcs[0].ntiles;

@@ -1,4 +1,4 @@
-"""The 32-pixel tile pass at the edges of its batches (64 particles), of its 8 x 8
+"""The tile pass at the edges of its batches (64 particles), of its 8 x 8
 blocks and of the image: list lengths around a batch and a work item, discs that
 just reach or miss a block, ragged image sides, against the FP64 oracle within
 the FP32 bar (1e-4)."""
@@ -46,21 +46,24 @@ def at_pixels(px, py, r, cam, rng):
             "I": rng.random(n), "s": rng.random(n)}
 
 
+@pytest.mark.parametrize("tile", [16, 32, 64])
 @pytest.mark.parametrize("n", [1, 2, 63, 64, 65, 127, 128, 129, 1023, 1024, 1025, 2100])
-def test_list_lengths(rnd, n):
+def test_list_lengths(rnd, n, tile):
     rng = np.random.default_rng(n)
     cam = scenes.camera(96, 64)
     p = at_pixels(rng.uniform(33, 63, n), rng.uniform(1, 31, n), rng.uniform(2.1, 12.0, n), cam, rng)
-    check(rnd, p, cam)
+    check(rnd, p, cam, tile_px=tile)
 
 
+@pytest.mark.parametrize("tile", [16, 32, 64])
 @pytest.mark.parametrize("w,h", [(1, 1), (7, 33), (33, 31), (40, 41), (65, 97)])
-def test_discs_at_block_edges_of_ragged_images(rnd, w, h):
+def test_discs_at_block_edges_of_ragged_images(rnd, w, h, tile):
     rng = np.random.default_rng(w * 100 + h)
     cam = scenes.camera(w, h)
     gx, gy = np.meshgrid(np.arange(-8, w + 9, 8), np.arange(-8, h + 9, 8))
     n = gx.size
     px, py = gx.ravel() + rng.normal(0, 0.02, n), gy.ravel() + rng.normal(0, 0.02, n)
-    for r in (2.05, 3.5, 7.99, 8.01, 30.0):
-        check(rnd, at_pixels(px, py, np.full(n, r), cam, rng), cam)
-    check(rnd, at_pixels(px, py, rng.uniform(2.1, 80.0, n), cam, rng), cam, mode=1, r_large=20.0)
+    for r in (0.3, 1.5, 2.05, 3.5, 7.99, 8.01, 30.0):
+        check(rnd, at_pixels(px, py, np.full(n, r), cam, rng), cam, tile_px=tile)
+    check(rnd, at_pixels(px, py, rng.uniform(0.2, 80.0, n), cam, rng), cam, mode=1, r_large=20.0,
+          tile_px=tile)
