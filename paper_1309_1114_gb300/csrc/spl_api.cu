@@ -540,15 +540,21 @@ static FrameConst make_frame(const spl_ctx *c, const spl_camera &cam) {
     for (int a = 0; a < 3; ++a) {
         double e = 0;
         for (int b = 0; b < 3; ++b) {
-            split_double(rows[a][b], fc.Rhi[3 * a + b], fc.Rlo[3 * a + b]);
+            float hi, lo;
+            split_double(rows[a][b], hi, lo);
+            (a == 0 ? fc.Rxy_hi[b].x : a == 1 ? fc.Rxy_hi[b].y : fc.Rz_hi[b]) = hi;
+            (a == 0 ? fc.Rxy_lo[b].x : a == 1 ? fc.Rxy_lo[b].y : fc.Rz_lo[b]) = lo;
             e += rows[a][b] * cam.eye[b];
         }
-        split_double(e, fc.Ehi[a], fc.Elo[a]);
+        split_double(e, a == 0 ? fc.Exy_hi.x : a == 1 ? fc.Exy_hi.y : fc.Ez_hi,
+                     a == 0 ? fc.Exy_lo.x : a == 1 ? fc.Exy_lo.y : fc.Ez_lo);
     }
     const double foc = 0.5 * cam.height / std::tan(0.5 * cam.fov_y_deg * M_PI / 180.0);
-    split_double(foc, fc.fhi, fc.flo);
-    fc.half_w = 0.5f * (float)cam.width;
-    fc.half_h = 0.5f * (float)cam.height;
+    float flo;
+    split_double(foc, fc.fhi, flo);
+    fc.f2_hi = make_float2(fc.fhi, -fc.fhi);
+    fc.f2_lo = make_float2(flo, -flo);
+    fc.half = make_float2(0.5f * (float)cam.width, 0.5f * (float)cam.height);
     fc.z_near = (float)cam.z_near;
     const spl_params &q = c->par;
     fc.sig_fac = (float)(q.sigma_per_h / q.s_box);
@@ -712,7 +718,7 @@ static void enqueue_binning(spl_ctx *c, const Views &vs, bool captured, cudaStre
     ra.ctab = c->ctab.p;
     ra.large_ids = c->large_ids.p;
     ra.st = c->dstats.p;
-    launch_raster(vs, ra, c->streaming ? c->chunk_attr : c->attr_type, s);
+    launch_raster(vs, ra, c->streaming ? c->chunk_attr : c->attr_type, c->sms, s);
     record_event(c, 1, s);
     BinArgs ba{};
     ba.recs = c->recs.p;
@@ -1562,7 +1568,7 @@ extern "C" int spl_render_noalloc(const spl_particles *p, const spl_camera *cam,
     ra.ctab = ctab;
     ra.large_ids = large_ids;
     ra.st = dst;
-    launch_raster(vs, ra, p->attr_type, s);
+    launch_raster(vs, ra, p->attr_type, sms, s);
     BinArgs ba{};
     ba.recs = recs;
     ba.large_ids = large_ids;

@@ -1,10 +1,40 @@
 // spl_geom.cuh -- device helpers shared by the rasteriser, the binning kernels
-// and the tile passes: record decoding and the tile footprint of a particle.
+// and the tile passes: packed FP32x2 arithmetic, record decoding and the tile footprint of a particle.
 #pragma once
 
 #include "spl_internal.cuh"
 
 namespace spl {
+
+// Two FP32 values in one 64-bit register pair: the operand of the packed
+// FP32x2 multiply and FMA (each half rounded as the scalar instruction).
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 pack2(float lo, float hi) {
+    f32x2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ void unpack2(f32x2 v, float &lo, float &hi) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+    f32x2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+    f32x2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ void fma2(f32x2 &acc, f32x2 a, f32x2 b) {
+    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc) : "l"(a), "l"(b));
+}
+__device__ __forceinline__ f32x2 fma2v(f32x2 a, f32x2 b, f32x2 c) {
+    f32x2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
 
 __device__ __forceinline__ int unpack_xi(float packed) {
     return (int)(short)(__float_as_uint(packed) & 0xFFFFu);
@@ -25,6 +55,13 @@ __device__ __forceinline__ int record_class(const FrameConst &fc, float r2) {
     return CLS_LARGE;
 }
 
+// sqrt(r^2) within 2^-22, far inside the margin of the box and disc tests below.
+__device__ __forceinline__ float approx_radius(float r2) {
+    float r;
+    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(r2));
+    return r;
+}
+
 // Pixel-centre bounding box of a splat, cut to the image: the pixels i with
 // |i + 1/2 - x_s| <= r (plus a margin of 1e-3 px + 1e-6 r, so that rounding
 // never drops a pixel that the exact clip test would keep).  Returns false
@@ -33,7 +70,7 @@ struct PixBox { int i0, i1, j0, j1; };
 
 __device__ __forceinline__ bool splat_box(const FrameConst &fc, float4 r0, float r2, PixBox &b) {
     const int xi = unpack_xi(r0.x), yi = unpack_yi(r0.x);
-    const float r = sqrtf(r2);
+    const float r = approx_radius(r2);
     const float m = r + 1e-3f + 1e-6f * r;
     // x_s - 1/2 relative to xi: xf - 1/2
     const float lo_x = (r0.y - 0.5f) - m, hi_x = (r0.y - 0.5f) + m;
@@ -50,7 +87,7 @@ __device__ __forceinline__ bool splat_box(const FrameConst &fc, float4 r0, float
 // Squared reach of a disc in the tile tests: the radius with the margin of
 // splat_box.
 __device__ __forceinline__ float disc_reach2(float r2) {
-    const float r = sqrtf(r2);
+    const float r = approx_radius(r2);
     const float m = r + 1e-3f + 1e-6f * r;
     return m * m;
 }

@@ -33,10 +33,13 @@ constexpr int kTileThreads = 256;        // 8 warps per tile CTA
 
 // Per-frame constants (camera in double-float: hi + lo pairs of FP32).
 struct FrameConst {
-    float Rhi[9], Rlo[9];      // rows right, up', fwd
-    float Ehi[3], Elo[3];      // R * eye
-    float fhi, flo;            // focal length
-    float half_w, half_h;
+    float2 Rxy_hi[3], Rxy_lo[3];   // columns of the rows (right, up')
+    float2 Exy_hi, Exy_lo;         // those rows times the eye
+    float2 f2_hi, f2_lo;           // focal length, (f, -f): y_s grows downwards
+    float2 half;                   // (width / 2, height / 2)
+    float Rz_hi[3], Rz_lo[3];      // row fwd
+    float Ez_hi, Ez_lo;
+    float fhi;                     // focal length rounded to float
     float z_near;
     float sig_fac;             // sigma_per_h / s_box
     float chi;
@@ -120,6 +123,18 @@ struct Segs {
 constexpr int kHashBits = 11;
 constexpr int kHash = 1 << kHashBits;
 constexpr int kChunk = 2048;
+// Sets that give the SMs less than kFewChunks CTAs of that size go through quarter
+// chunks with quarter tables: a CTA takes its chunk 256 particles at a time, so that a
+// longer chunk is a longer chain (200k particles: raster 0.032 -> 0.022, lists 0.043 ->
+// 0.029 ms; 1.3M: 0.107 -> 0.087, 0.163 -> 0.113). On larger sets the four times as many
+// tables cost more (10M: raster 0.369 -> 0.588 ms; the two meet near 3M).
+struct BinShape {
+    int chunk, hash_bits;
+};
+constexpr int kFewChunks = 10;
+__host__ __device__ inline BinShape bin_shape(int64_t n, int sms) {
+    return n < (int64_t)sms * kFewChunks * kChunk ? BinShape{kChunk / 4, kHashBits - 2} : BinShape{kChunk, kHashBits};
+}
 __host__ __device__ constexpr int64_t ctab_entries(int64_t n, int nviews) {
     return ((n + kChunk - 1) / kChunk > 0 ? (n + kChunk - 1) / kChunk : 1) *
            (nviews > 0 ? nviews : 1) * kHash;
@@ -147,6 +162,7 @@ struct RasterArgs {
     int2 *ctab;                // per (CTA, view): the CTA hash table, (slot, offset in the slot)
     unsigned *large_ids;       // record indices, capacity nviews * n
     DevStats *st;
+    BinShape shape;
 };
 
 // A list slot's range [offsets[k], offsets[k+1]) holds first the entries
@@ -165,6 +181,7 @@ struct BinArgs {
     unsigned *entries;         // record indices
     int64_t entries_cap;
     DevStats *st;
+    BinShape shape;
 };
 
 struct TileArgs {
@@ -191,7 +208,7 @@ constexpr int kNParam = kHid * kFeat + 2 * kHid + 1;
 // Launchers (stream-ordered, no synchronisation).  Every count the kernels
 // need after binning (entries, work items) is read from device memory, so
 // the whole sequence can be captured in a CUDA graph.
-void launch_raster(const Views &v, const RasterArgs &a, int attr, cudaStream_t s);
+void launch_raster(const Views &v, RasterArgs a, int attr, int sms, cudaStream_t s);
 void launch_count_large(const Views &v, const BinArgs &a, int sms, cudaStream_t s);
 
 // The start of a frame: zeroes the slot counts and the frame's statistics; a single
@@ -231,7 +248,7 @@ struct ListArgs {
     float *const *images;
     int large_blocks, item_blocks, zero_blocks;
 };
-void launch_lists(const Views &v, const BinArgs &a, ListArgs l, bool zero, int sms, cudaStream_t s);
+void launch_lists(const Views &v, BinArgs a, ListArgs l, bool zero, int sms, cudaStream_t s);
 void launch_tile_pass(const Views &v, const TileArgs &a, int sms, cudaStream_t s);
 void launch_large_pass(const Views &v, const TileArgs &a, int sms, cudaStream_t s);
 // Absorption mode: the depth-ordered pass and the composition of split tiles.

@@ -1,6 +1,6 @@
-// spl_tile.cuh -- the band geometry of a tile CTA and the packed FP32x2
-// helpers shared by the additive passes (spl_tile.cu) and the general
-// absorption pass (spl_absorb.cu).
+// spl_tile.cuh -- shared-memory access by address for the additive passes
+// (spl_tile.cu), and the band geometry of the general absorption pass
+// (spl_absorb.cu).
 #pragma once
 #include "spl_geom.cuh"
 
@@ -28,36 +28,6 @@ struct Shape {
     // particles that a half-warp's 64-bit stores reach in different banks
     static constexpr int WXS = T + 8;
 };
-
-// Two FP32 values in one 64-bit register pair: the operand of the packed
-// FP32x2 multiply and FMA (each half rounded as the scalar instruction).
-typedef unsigned long long f32x2;
-__device__ __forceinline__ f32x2 pack2(float lo, float hi) {
-    f32x2 r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-    return r;
-}
-__device__ __forceinline__ void unpack2(f32x2 v, float &lo, float &hi) {
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
-}
-__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
-    f32x2 r;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
-    f32x2 r;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ void fma2(f32x2 &acc, f32x2 a, f32x2 b) {
-    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc) : "l"(a), "l"(b));
-}
-__device__ __forceinline__ f32x2 fma2v(f32x2 a, f32x2 b, f32x2 c) {
-    f32x2 r;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-    return r;
-}
 
 // Shared memory by 32-bit address, and 16-byte asynchronous copies into it.
 __device__ __forceinline__ float4 lds4(unsigned a) {
