@@ -97,7 +97,7 @@ struct spl_ctx {
     DevBuf<unsigned> rank;
     DevBuf<int> sort_hist;
     DevBuf<float4> partial;
-    DevBuf<int> counts, ovf;
+    DevBuf<int> counts, ovf, full;
     DevBuf<int2> ctab;
     DevBuf<long long> offsets, cursor;
     DevBuf<unsigned> large_ids, entries;
@@ -280,7 +280,7 @@ extern "C" int spl_destroy(spl_ctx *c) {
     c->rec2.release(); c->pkeys.release(); c->ptmp.release(); c->ekeys.release();
     c->etmp.release(); c->rank.release(); c->sort_hist.release(); c->partial.release();
     c->counts.release(); c->offsets.release(); c->cursor.release();
-    c->ovf.release(); c->ctab.release();
+    c->ovf.release(); c->ctab.release(); c->full.release();
     c->large_ids.release(); c->entries.release(); c->dstats.release();
     c->item_counts.release(); c->item_offsets.release(); c->items.release();
     c->slot_part.release();
@@ -634,6 +634,7 @@ static int prepare_views(spl_ctx *c, const spl_camera *cams, int V, float *const
     SPL_TRY(grow(c, c->large_ids, recs ? recs : 1));
     SPL_TRY(grow(c, c->counts, (size_t)NLIST * tiles));
     SPL_TRY(grow(c, c->ovf, (size_t)NLIST * tiles));
+    SPL_TRY(grow(c, c->full, (size_t)tiles));
     SPL_TRY(grow(c, c->ctab, (size_t)ctab_entries(src_n(c), V)));
     SPL_TRY(grow(c, c->offsets, (size_t)NLIST * tiles + 1));
     SPL_TRY(grow(c, c->cursor, (size_t)NLIST * tiles));
@@ -679,6 +680,7 @@ static void enqueue_binning(spl_ctx *c, const Views &vs, bool captured, cudaStre
     SetupArgs sa{};
     sa.counts = c->counts.p;
     sa.ovf = c->ovf.p;
+    sa.full = c->full.p;
     sa.slots = NLIST * vs.total_tiles;
     sa.st = c->dstats.p;
     if (captured || vs.nviews > 1) {
@@ -745,6 +747,7 @@ static void enqueue_lists(spl_ctx *c, const Views &vs, cudaStream_t s) {
     ba.offsets = c->offsets.p;
     ba.ctab = c->ctab.p;
     ba.cursor = c->cursor.p;
+    ba.full = c->full.p;
     ba.entries = c->entries.p;
     ba.entries_cap = (int64_t)c->entries.cap;
     ba.st = c->dstats.p;
@@ -759,6 +762,8 @@ static void enqueue_passes(spl_ctx *c, const Views &vs, bool large_pass, cudaStr
     ta.offsets = c->offsets.p;
     ta.entries = c->entries.p;
     ta.entries_cap = (long long)c->entries.cap;
+    ta.full = c->full.p;
+    ta.cover = cover_pays(c->hstats->totals[L_LARGE], vs.total_tiles, vs.tile);
     ta.items = c->items.p;
     ta.items_cap = (int)c->items.cap;
     ta.images = c->d_images.p;
@@ -861,7 +866,7 @@ static int render_views(spl_ctx *c, const spl_camera *cams, int V, float *const 
         SPL_TRY(grow(c, c->entries, (size_t)(total ? total : 1)));
         SPL_TRY(grow(c, c->items, (size_t)(n_tile_items + n_large_items + 1)));
         SPL_CUDA(cudaMemsetAsync(&c->dstats.p->err, 0, sizeof(unsigned), s));
-        launch_slot_cursor(NLIST * vs.total_tiles, c->counts.p, c->offsets.p, c->cursor.p, s);
+        launch_slot_cursor(NLIST * vs.total_tiles, c->counts.p, c->offsets.p, c->cursor.p, c->full.p, s);
         enqueue_lists(c, vs, s);
         SPL_CUDA(cudaGetLastError());
     }
@@ -1444,7 +1449,8 @@ constexpr size_t kNaView = kNaItems + na_round(sizeof(WorkItem) * kNaMaxItems);
 constexpr size_t kNaImage = kNaView + na_round(sizeof(FrameConst));
 constexpr size_t kNaPart = kNaImage + na_round(sizeof(float *));
 constexpr size_t kNaParts = 64;     // at least slot_parts(kNaMaxTiles)
-constexpr size_t kNaBytes = kNaPart + na_round(sizeof(long long) * kNaParts);
+constexpr size_t kNaFull = kNaPart + na_round(sizeof(long long) * kNaParts);
+constexpr size_t kNaBytes = kNaFull + na_round(sizeof(int) * kNaMaxTiles);
 }  // namespace
 
 static_assert(kNaBytes < ((size_t)17 << 20), "the fixed scratch stays below 17 MiB");
@@ -1536,6 +1542,7 @@ extern "C" int spl_render_noalloc(const spl_particles *p, const spl_camera *cam,
     float **d_img = reinterpret_cast<float **>(base + kNaImage);
     long long *part = reinterpret_cast<long long *>(base + kNaPart);
     if (slot_parts(fc.ntiles) > kNaParts) return SPL_ELIMIT;
+    int *full = reinterpret_cast<int *>(base + kNaFull);
     int sms = 1;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
     FrameConst fcv = fc;
@@ -1554,7 +1561,7 @@ extern "C" int spl_render_noalloc(const spl_particles *p, const spl_camera *cam,
     // (the error word stays: the previous call's passes may have set it, and
     // it is read at this call's synchronisation point)
     SPL_CUDA(cudaMemcpyAsync(pal, rgb, sizeof(float) * 3 * npal, cudaMemcpyHostToDevice, s));
-    launch_setup(SetupArgs{fcv, d_image, d_fc, d_img, counts, ovf, NLIST * fc.ntiles, dst}, sms, s);
+    launch_setup(SetupArgs{fcv, d_image, d_fc, d_img, counts, ovf, full, NLIST * fc.ntiles, dst}, sms, s);
     RasterArgs ra{};
     ra.n = p->n;
     ra.x = p->x; ra.y = p->y; ra.z = p->z;
@@ -1596,6 +1603,7 @@ extern "C" int spl_render_noalloc(const spl_particles *p, const spl_camera *cam,
     const int n_tile_items = h.item_totals[0], n_large_items = h.item_totals[1];
     if (total > kNaMaxEntries || (int64_t)n_tile_items + n_large_items > kNaMaxItems)
         return SPL_ELIMIT;
+    ba.full = full;
     ba.entries = entries;
     ba.entries_cap = kNaMaxEntries;
     launch_lists(vs, ba, ListArgs{item_offsets, items, kNaMaxItems, seg, d_img, 0, 0, 0}, true, sms, s);
@@ -1604,6 +1612,8 @@ extern "C" int spl_render_noalloc(const spl_particles *p, const spl_camera *cam,
     ta.offsets = offsets;
     ta.entries = entries;
     ta.entries_cap = kNaMaxEntries;
+    ta.full = full;
+    ta.cover = cover_pays(h.totals[L_LARGE], fc.ntiles, fc.tile);
     ta.items = items;
     ta.items_cap = kNaMaxItems;
     ta.images = d_img;

@@ -107,6 +107,19 @@ __device__ __forceinline__ bool disc_meets_tile(const FrameConst &fc, float4 r0,
     return dx * dx + dy * dy <= reach2;
 }
 
+// Does a disc of squared radius r2 cover every pixel centre of tile (tx, ty), far enough
+// from its edge that every clip factor is exactly 1?
+__device__ __forceinline__ bool disc_covers_tile(const FrameConst &fc, float4 r0, float r2, int tx, int ty) {
+    const int xi = unpack_xi(r0.x), yi = unpack_yi(r0.x);
+    const float ax = (float)(tx * fc.tile - xi) + 0.5f - r0.y;
+    const float bx = (float)(min((tx + 1) * fc.tile, fc.width) - 1 - xi) + 0.5f - r0.y;
+    const float ay = (float)(ty * fc.tile - yi) + 0.5f - r0.z;
+    const float by = (float)(min((ty + 1) * fc.tile, fc.height) - 1 - yi) + 0.5f - r0.z;
+    const float dx = fmaxf(-ax, bx), dy = fmaxf(-ay, by);
+    const float r = approx_radius(r2), m = r - 1e-3f - 4e-6f * r;
+    return m > 0.f && dx * dx + dy * dy <= m * m;
+}
+
 // exp(-d2/sigma^2) = 2^(-kq d2) with the hardware exp2 (PTX ex2.approx.ftz.f32,
 // maximum relative error about 2^-22 over the range used here).
 __device__ __forceinline__ float ex2_neg(float kq_d2) {

@@ -501,8 +501,12 @@ __device__ __forceinline__ void large_tiles(const Views &vs, const BinArgs &a, u
             if (MODE == 0) {
                 atomicAdd(&a.ovf[slot], 1);
             } else {
+                // the entries that cover their tile go to the list's end (16-pixel
+                // tiles have no use for them)
+                const bool full = fc.tile > 16 && disc_covers_tile(fc, r0, r1.x, tx, ty);
                 const long long pos =
-                    (long long)atomicAdd(reinterpret_cast<unsigned long long *>(&a.cursor[slot]), 1ULL);
+                    full ? a.offsets[slot + 1] - 1 - atomicAdd(&a.full[fc.tile_base + ty * fc.ntx + tx], 1)
+                         : (long long)atomicAdd(reinterpret_cast<unsigned long long *>(&a.cursor[slot]), 1ULL);
                 if (pos < a.entries_cap)
                     a.entries[pos] = rec;
                 else
@@ -523,9 +527,11 @@ void launch_count_large(const Views &vs, const BinArgs &a, int sms, cudaStream_t
 }
 
 __global__ void slot_cursor_kernel(int m, const int *counts, const long long *offsets,
-                                   long long *cursor) {
-    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < m; k += gridDim.x * blockDim.x)
+                                   long long *cursor, int *full) {
+    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < m; k += gridDim.x * blockDim.x) {
         cursor[k] = offsets[k] + counts[k];
+        if (k < m / NLIST) full[k] = 0;
+    }
 }
 
 // Exclusive scan of one value per thread over a block of 1024 threads (wsum: 33).
@@ -582,10 +588,10 @@ void launch_scan(int m, const int *in, int *out, cudaStream_t s) {
 }
 
 void launch_slot_cursor(int m, const int *counts, const long long *offsets, long long *cursor,
-                        cudaStream_t s) {
+                        int *full, cudaStream_t s) {
     const int grid = (m + 255) / 256 < 1024 ? (m + 255) / 256 : 1024;
     if (grid <= 0) return;
-    slot_cursor_kernel<<<grid, 256, 0, s>>>(m, counts, offsets, cursor);
+    slot_cursor_kernel<<<grid, 256, 0, s>>>(m, counts, offsets, cursor, full);
     ++g_launches;
 }
 
@@ -625,7 +631,10 @@ __device__ __forceinline__ Segs frame_segs(const unsigned long long *tot, int sm
         if (sms > 0) {
             len = (long long)((l == L_LARGE ? tot[L_LARGE] : work) / (unsigned long long)(8 * sms));
             len = (len + 63) / 64 * 64;
-            len = len < whole / kSegShrink ? whole / kSegShrink : (len > whole ? whole : len);
+            // longer large segments where there are plenty: fewer partial tiles (100M
+            // heavy-tailed particles, large pass 3.71 -> 3.44 ms; 8 times: the same)
+            const int most = l == L_LARGE ? 4 * whole : whole;
+            len = len < whole / kSegShrink ? whole / kSegShrink : (len > most ? most : len);
         }
         segs.len[l] = (int)(full[l] / whole * len);
     }
@@ -997,6 +1006,7 @@ __global__ void __launch_bounds__(256) setup_kernel(const __grid_constant__ Setu
     for (int k = i; k < a.slots; k += stride) {
         a.counts[k] = 0;
         a.ovf[k] = 0;
+        if (k < a.slots / NLIST) a.full[k] = 0;
     }
     if (i < (int)(offsetof(DevStats, err) / sizeof(int))) reinterpret_cast<int *>(a.st)[i] = 0;
     if (a.fcs) {

@@ -29,7 +29,8 @@
 //     writes its pixels once.
 // The large pass (r > r_large, Sec. 4.3) runs after the tile pass with the
 // same scheme over segments of the tiles' large lists and adds its partial
-// tiles into the image.
+// tiles into the image; tiles that lie wholly inside a disc go through the
+// covering pass.
 //
 // Clip (Eq. 2: zero beyond chi*sigma).  With B = 2^20 / r^2 the tables hold
 // dx^2 * B per column and (r^2 - dy^2) * B + 1 per row; the clip factor is
@@ -379,6 +380,17 @@ __device__ __forceinline__ void shared_lists(const FrameConst &fc, const TileArg
     }
 }
 
+// The entries of a large item that cover its whole tile: the last ones of the tile's
+// list, from the first result to the second.  They go through the covering pass, unless
+// they are too few to be worth a start there.
+constexpr int kFewFull = 64;
+__device__ __forceinline__ long long item_full_start(const TileArgs &a, const FrameConst &fc,
+                                                     const WorkItem &w) {
+    const int slot = fc.slot_base + L_LARGE * fc.ntiles + w.tile - fc.tile_base;
+    const long long from = max(w.start, a.offsets[slot + 1] - a.full[w.tile]);
+    return w.end - from < kFewFull ? w.end : from;
+}
+
 // Persistent pass over the work items of every view of the batch: the tile
 // pass takes items [0, item_totals[0]), the large pass the next
 // item_totals[1] (both counts read from device memory).
@@ -433,7 +445,8 @@ __global__ void __launch_bounds__(kTileThreads, kItemCtas) item_kernel(Views vs,
         // the entries written
         const bool mine = list < 0 || list >= L_MEDIUM;
         const long long lb2 = min(w.start, cap);
-        const int n2 = mine ? (int)(min(w.end, cap) - lb2) : 0;
+        const long long last = LARGE && T > 16 && a.cover ? item_full_start(a, fc, w) : w.end;
+        const int n2 = mine ? (int)(min(last, cap) - lb2) : 0;
         float quad[2][2][3];
         quad_list<W, (SUB > 1)>(a, a.entries + lb2, n2, x0, y0,
                                 (unsigned)__cvta_generic_to_shared(smem_raw), quad);
@@ -537,6 +550,229 @@ __global__ void __launch_bounds__(kTileThreads, kItemCtas) item_kernel(Views vs,
     }
 }
 
+// ---------------------------------------------------------------------------
+// The covering pass: large particles over tiles that lie wholly inside their discs (most
+// tiles of a particle much wider than a tile).  No clip, and every pixel is covered, so
+// that a lane can hold 4 x 4 pixels and a warp half the tile: per particle a warp loads four
+// column weights and four rows' terms (10 wavefronts per 512 pixels, where the blocks of
+// the tile pass take 26) and adds 48 products per lane.  The two warps of a tile are
+// repeated four times over the particles.  16 warps per SM leave it bound by latency
+// (FMA pipe 40 %, 50 cycles per entry and SM where the tile pass took 78).  Large pass of
+// the 100M heavy-tailed frame 4.96 -> 3.44 ms, of 1M particles in six orbit views 6.89 ->
+// 5.33 ms.
+// ---------------------------------------------------------------------------
+struct Cover {
+    static constexpr int P = 64;
+    // one particle's tables: 32 column weights, 16 row pairs (e_R w_a, e_R w_b, e_G w_a,
+    // e_G w_b), 16 row pairs (e_B w_a, e_B w_b); padding and slot order as in Quad
+    static constexpr int ROWA = 128, ROWB = 384, BYTES = 544;
+    __device__ static __forceinline__ unsigned slot(int p) {
+        return (unsigned)((p & ~3) | ((p & 1) << 1) | ((p >> 1) & 1));
+    }
+    static constexpr int kStage = P * BYTES;
+    static constexpr int kSmem = kStage + 2 * P * 32;
+    static constexpr int kTile = 3 * 32 * 32;      // floats; two tiles reuse the tables
+    static_assert(2 * 4 * kTile <= kStage, "the tables hold two tiles");
+};
+constexpr int kCoverCtas = 2, kCoverUnroll = 2;   // 128 registers (3 CTAs at 80 spill: 7 % longer)
+
+template <int T>
+__global__ void __launch_bounds__(kTileThreads, kCoverCtas) cover_kernel(Views vs, TileArgs a) {
+    constexpr int W = 32, SIDE = T / W, SUB = SIDE * SIDE, P = Cover::P;
+    extern __shared__ float4 smem_raw[];
+    __shared__ int s_item[2];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const unsigned smem = (unsigned)__cvta_generic_to_shared(smem_raw);
+    float *tiles = reinterpret_cast<float *>(smem_raw);
+    int *counter = &a.st->item_counter[2];
+    const int item0 = a.st->item_totals[0];
+    const int n_work = min(a.st->item_totals[1], a.items_cap - item0) * SUB;
+    // this lane's pixels: columns 4 cg .. 4 cg + 3, row pairs rg and rg + 1
+    const int cg = lane & 7, rg = (warp & 1) * 8 + (lane >> 3) * 2, group = warp >> 1;
+    const unsigned at0 = smem + Cover::slot(group) * Cover::BYTES;
+    const unsigned col_at = at0 + 16u * cg, row_at = at0 + Cover::ROWA + 16u * rg;
+    const unsigned blue_at = at0 + Cover::ROWB + 8u * rg;
+    const int sp = tid >> 1;
+    const unsigned half = (unsigned)(tid & 1);
+    const unsigned stage = smem + Cover::kStage, stage_at = stage + half * (P * 16) + (unsigned)sp * 16u;
+    // where there are few items most have nothing for this pass: eight at a time, one
+    // lane each
+    const int step = n_work < 8 * (int)gridDim.x ? 8 : 1;
+    __shared__ unsigned s_some;
+    int next = 0;
+    unsigned some = 0;                     // items of the current step still to be done
+    if (tid == 0) s_item[0] = atomicAdd(counter, step);
+    for (int turn = 0, it0 = 0;;) {
+        __syncthreads();
+        if (!some) {
+            it0 = s_item[turn];
+            if (it0 >= n_work) break;
+            turn ^= 1;
+            if (tid == 0) next = atomicAdd(counter, step);
+            if (warp == 0) {
+                bool has = lane < step && it0 + lane < n_work;
+                if (has) {
+                    const WorkItem w = a.items[item0 + (it0 + lane) / SUB];
+                    has = item_full_start(a, vs.fcs[item_view(w)], w) < w.end;
+                }
+                const unsigned m = __ballot_sync(0xffffffffu, has);
+                if (lane == 0) {
+                    s_some = m;
+                    s_item[turn] = next;
+                }
+            }
+            __syncthreads();
+            some = s_some;
+            if (!some) continue;
+        }
+        const int it = it0 + __ffs(some) - 1;
+        some &= some - 1u;
+        const int idx = item0 + it / SUB, sub = it % SUB;
+        const WorkItem w = a.items[idx];
+        const FrameConst &fc = vs.fcs[item_view(w)];
+        const int tile = w.tile - fc.tile_base;
+        const int x0 = (tile % fc.ntx) * T + sub % SIDE * W, y0 = (tile / fc.ntx) * T + sub / SIDE * W;
+        const long long lb = item_full_start(a, fc, w);
+        int n = (int)(min(w.end, a.entries_cap) - lb);
+        if (x0 >= fc.width || y0 >= fc.height) n = 0;
+        if (n > 0) {
+            const long long t_start = clock64();
+            const unsigned *ent = a.entries + lb;
+            f32x2 acc[2][4][3];
+#pragma unroll
+            for (int m = 0; m < 2; ++m)
+#pragma unroll
+                for (int k = 0; k < 4; ++k) acc[m][k][0] = acc[m][k][1] = acc[m][k][2] = 0ull;
+            unsigned id = 0;
+            if (sp < P && sp < n) {
+                cp_async16(stage_at, reinterpret_cast<const char *>(a.recs + ent[sp]) + half * 16);
+                if (P + sp < n) id = ent[P + sp];
+            }
+            unsigned buf = 0;
+#pragma unroll 1
+            for (int base = 0; base < n; base += P) {
+                const int cnt = n - base < P ? n - base : P;
+                const unsigned st = stage + buf * (P * 32);
+                cp_async_wait();
+                __syncthreads();
+                if (sp < P && base + P + sp < n) {
+                    cp_async16(stage_at + (buf ^ 1u) * (P * 32),
+                               reinterpret_cast<const char *>(a.recs + id) + half * 16);
+                    if (base + 2 * P + sp < n) id = ent[base + 2 * P + sp];
+                }
+                const int p = tid >> 2, q = tid & 3;
+                if (p < cnt) {
+                    // thread q of a particle's four: pairs q, q + 4, q + 8, q + 12 of columns and rows
+                    const float4 r0 = lds4(st + p * 16), r1 = lds4(st + P * 16 + p * 16);
+                    const f32x2 nkq = pack2(-r0.w, -r0.w);
+                    const float xf = (float)(x0 - unpack_xi(r0.x) + 2 * q);
+                    const float yf = (float)(y0 - unpack_yi(r0.x) + 2 * q);
+                    const f32x2 xh = pack2(0.5f - r0.y, 0.5f - r0.y), yh = pack2(0.5f - r0.z, 0.5f - r0.z);
+                    const f32x2 er = pack2(r1.y, r1.y), eg = pack2(r1.z, r1.z), eb = pack2(r1.w, r1.w);
+                    const unsigned tab = smem + Cover::slot(p) * Cover::BYTES;
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        const f32x2 dx = add2(pack2(xf + 8.f * u, xf + 8.f * u + 1.f), xh);
+                        const f32x2 dy = add2(pack2(yf + 8.f * u, yf + 8.f * u + 1.f), yh);
+                        float ta, tb, wa, wb;
+                        unpack2(mul2(mul2(dx, dx), nkq), ta, tb);
+                        asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(wa) : "f"(ta));
+                        asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(wb) : "f"(tb));
+                        sts2(tab + 8 * q + 32 * u, pack2(wa, wb));
+                        unpack2(mul2(mul2(dy, dy), nkq), ta, tb);
+                        asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(wa) : "f"(ta));
+                        asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(wb) : "f"(tb));
+                        const f32x2 wy = pack2(wa, wb);
+                        sts2x2(tab + Cover::ROWA + 16 * q + 64 * u, mul2(er, wy), mul2(eg, wy));
+                        sts2(tab + Cover::ROWB + 8 * q + 32 * u, mul2(eb, wy));
+                    }
+                }
+                __syncthreads();
+                unsigned off = 0;
+#pragma unroll kCoverUnroll
+                for (int i = group; i < cnt; i += 4, off += 4 * Cover::BYTES) {
+                    const float4 c = lds4(col_at + off);
+                    f32x2 er0, eg0, er1, eg1, eb0, eb1;
+                    lds2x2(row_at + off, er0, eg0);
+                    lds2x2(row_at + off + 16, er1, eg1);
+                    lds2x2(blue_at + off, eb0, eb1);
+                    const float wx[4] = {c.x, c.y, c.z, c.w};
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        const f32x2 wk = pack2(wx[k], wx[k]);
+                        fma2(acc[0][k][0], er0, wk);
+                        fma2(acc[0][k][1], eg0, wk);
+                        fma2(acc[0][k][2], eb0, wk);
+                        fma2(acc[1][k][0], er1, wk);
+                        fma2(acc[1][k][1], eg1, wk);
+                        fma2(acc[1][k][2], eb1, wk);
+                    }
+                }
+                buf ^= 1u;
+            }
+            // the four groups' sums: 2 and 3 through shared memory to 0 and 1, then 1 to 0,
+            // whose sum every thread writes
+            auto exchange = [&](float *t, bool put) {
+#pragma unroll
+                for (int m = 0; m < 2; ++m)
+#pragma unroll
+                    for (int c = 0; c < 3; ++c)
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) {
+                            float *d = t + (c * W + 2 * (rg + m)) * W + 4 * cg + k;
+                            float lo, hi;
+                            unpack2(acc[m][k][c], lo, hi);
+                            if (put) {
+                                d[0] = lo;
+                                d[W] = hi;
+                            } else {
+                                acc[m][k][c] = pack2(lo + d[0], hi + d[W]);
+                            }
+                        }
+            };
+            __syncthreads();
+            if (group >= 2) exchange(tiles + (group - 2) * Cover::kTile, true);
+            __syncthreads();
+            if (group < 2) exchange(tiles + group * Cover::kTile, false);
+            if (group == 1) exchange(tiles + Cover::kTile, true);
+            __syncthreads();
+            if (group == 0) {
+                exchange(tiles + Cover::kTile, false);
+                exchange(tiles, true);
+            }
+            __syncthreads();
+            const bool sole = item_sole(w);
+            float *image = a.images[item_view(w)];
+            // 12 values per thread, every load before the first store
+            constexpr int PER = Cover::kTile / kTileThreads;
+            float v[PER];
+#pragma unroll
+            for (int u = 0; u < PER; ++u) {
+                const int k = tid + u * kTileThreads, row = k / (3 * W), x3 = k % (3 * W);
+                v[u] = tiles[(x3 % 3 * W + row) * W + x3 / 3];
+                if (sole && y0 + row < fc.height && x0 + x3 / 3 < fc.width)
+                    v[u] += image[(int64_t)3 * fc.width * (y0 + row) + 3 * x0 + x3];
+            }
+#pragma unroll
+            for (int u = 0; u < PER; ++u) {
+                const int k = tid + u * kTileThreads, row = k / (3 * W), x3 = k % (3 * W);
+                if (y0 + row < fc.height && x0 + x3 / 3 < fc.width)
+                    put_value(image + (int64_t)3 * fc.width * (y0 + row) + 3 * x0 + x3, v[u], sole);
+            }
+            if (a.item_cycles && tid == 0)
+                atomicAdd(reinterpret_cast<unsigned long long *>(&a.item_cycles[idx]),
+                          (unsigned long long)(clock64() - t_start));
+        }
+    }
+}
+
+template <int T>
+static void launch_cover_t(const Views &vs, const TileArgs &a, int sms, cudaStream_t s) {
+    cudaFuncSetAttribute(cover_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cover::kSmem);
+    cover_kernel<T><<<sms * kCoverCtas, kTileThreads, Cover::kSmem, s>>>(vs, a);
+    ++g_launches;
+}
+
 template <int T, bool LARGE>
 static void launch_items_t(const Views &vs, const TileArgs &a, int sms, cudaStream_t s) {
     constexpr size_t bytes = Quad<(T == 16 ? 16 : 32)>::kSmem;
@@ -562,6 +798,11 @@ void launch_tile_pass(const Views &vs, const TileArgs &a, int sms, cudaStream_t 
 
 void launch_large_pass(const Views &vs, const TileArgs &a, int sms, cudaStream_t s) {
     launch_items<true>(vs, a, sms, s);
+    if (!a.cover) return;
+    if (vs.tile == 32)
+        launch_cover_t<32>(vs, a, sms, s);
+    else if (vs.tile == 64)
+        launch_cover_t<64>(vs, a, sms, s);
 }
 
 // E_p = A_p solution of Eq. 1 applied to the additive sum: I = 1 - exp(-S).

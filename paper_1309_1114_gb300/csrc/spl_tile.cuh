@@ -48,6 +48,9 @@ __device__ __forceinline__ uint4 ldsu4(unsigned a) {
 __device__ __forceinline__ void sts2x2(unsigned a, f32x2 u, f32x2 v) {
     asm volatile("st.shared.v2.b64 [%0], {%1, %2};" ::"r"(a), "l"(u), "l"(v) : "memory");
 }
+__device__ __forceinline__ void sts2(unsigned a, f32x2 u) {
+    asm volatile("st.shared.b64 [%0], %1;" ::"r"(a), "l"(u) : "memory");
+}
 __device__ __forceinline__ unsigned lds_u8(unsigned a) {
     unsigned v;
     asm volatile("ld.shared.u8 %0, [%1];" : "=r"(v) : "r"(a));
