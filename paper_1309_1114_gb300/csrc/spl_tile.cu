@@ -131,8 +131,8 @@ __device__ __forceinline__ void warp_points(const TileArgs &a, bool valid, float
 // ---------------------------------------------------------------------------
 //
 // W is the side of the pixels a CTA works on: 32 for 32-pixel tiles (8 warps, 16 blocks);
-// a 64-pixel tile is four such parts, each its own piece of work over the same lists
-// (particles that miss the part are not tabulated); 16 for 16-pixel tiles, whose two
+// a 64-pixel tile is four such parts, each its own piece of work over the same list
+// (particles that miss the part are not tabulated), added to the image by atomics; 16 for 16-pixel tiles, whose two
 // pairs of blocks are shared by four warps each, a warp taking 16 of a batch's 64
 // particles.  A lane per pixel over 16 x 2 bands (16), and 64 x 8 bands with 128
 // registers (64), took 7.98 and 8.69 ms on the clustered 10M / 1024^2 frame; these
@@ -161,6 +161,7 @@ struct Quad {
     // sums, reuse the tables
     static constexpr int kPart = 12 * W * W;
     static_assert(kPart + (G > 1 ? G * 12 * W * W : 0) <= kNone, "the tables hold both");
+    static_assert(W == 16 || 12 * 64 * 64 <= kNone, "the tables hold a 64-pixel tile");
 };
 
 // Tabulate particle (r0, r1) into the block tab: thread q of its four fills
@@ -396,9 +397,54 @@ __device__ __forceinline__ long long item_full_start(const TileArgs &a, const Fr
 // item_totals[1] (both counts read from device memory).
 constexpr int kItemCtas = 4;      // per SM: 64 registers, 56 KB of shared memory at W = 32
 
+// Points and small particles of an item of a 64-pixel tile, over the whole tile: each of its
+// four parts going through these lists cost more than it shared (7.9M points and
+// small particles on 195 x 89: tile pass 0.394 ms, 0.299 so).
+__device__ __forceinline__ void whole_tile_lists(const Views &vs, const TileArgs &a, const WorkItem &w,
+                                                 const FrameConst &fc, int tx0, int ty0,
+                                                 float (*sacc)[64][64]) {
+    const int list = item_list(w), tid = threadIdx.x;
+    const long long cap = a.entries_cap;
+    long long lb0 = 0, le0 = 0, lb1 = 0, le1 = 0;
+    if (list < 0) {
+        const long long *o = a.offsets + fc.slot_base + w.tile - fc.tile_base;
+        lb0 = min(o[L_POINT * fc.ntiles], cap); le0 = min(o[L_POINT * fc.ntiles + 1], cap);
+        lb1 = min(o[L_SMALL * fc.ntiles], cap); le1 = min(o[L_SMALL * fc.ntiles + 1], cap);
+    } else if (list == L_POINT) {
+        lb0 = min(w.start, cap); le0 = min(w.end, cap);
+    } else if (list == L_SMALL) {
+        lb1 = min(w.start, cap); le1 = min(w.end, cap);
+    }
+    if (le0 <= lb0 && le1 <= lb1) return;
+    for (int k = tid; k < 3 * 64 * 64; k += kTileThreads) (&sacc[0][0][0])[k] = 0.f;
+    __syncthreads();
+    shared_lists<64, 64>(fc, a, lb0, le0, lb1, le1, tx0, ty0, tx0, ty0, sacc, tid, kTileThreads);
+    __syncthreads();
+    float *image = a.images[item_view(w)];
+    for (int k = tid; k < 3 * 64 * 64; k += kTileThreads) {
+        const int row = k / 192, x3 = k % 192;
+        if (ty0 + row < fc.height && tx0 + x3 / 3 < fc.width)
+            put_value(image + (int64_t)3 * fc.width * (ty0 + row) + 3 * tx0 + x3, sacc[x3 % 3][row][x3 / 3],
+                      false);
+    }
+}
+
+// The cycles of an item, when they are recorded (zeroed by the caller; the parts of a tile
+// add up).
+__device__ __forceinline__ void finish(const TileArgs &a, int idx, long long t_start) {
+    if (!a.item_cycles) return;
+    __syncthreads();
+    if (threadIdx.x == 0)
+        atomicAdd(reinterpret_cast<unsigned long long *>(&a.item_cycles[idx]),
+                  (unsigned long long)(clock64() - t_start));
+}
+
 template <int T, bool LARGE>
 __global__ void __launch_bounds__(kTileThreads, kItemCtas) item_kernel(Views vs, TileArgs a) {
-    constexpr int W = T == 16 ? 16 : 32, SIDE = T / W, SUB = SIDE * SIDE;
+    // a 64-pixel tile: four parts for its medium (large) particles, and in the tile pass a
+    // fifth for its points and small particles, over the whole tile
+    constexpr int W = T == 16 ? 16 : 32, SIDE = T / W;
+    constexpr int SUB = SIDE * SIDE + (T == 64 && !LARGE ? 1 : 0);
     using Q = Quad<W>;
     extern __shared__ float4 smem_raw[];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -439,6 +485,14 @@ __global__ void __launch_bounds__(kTileThreads, kItemCtas) item_kernel(Views vs,
         const int x0 = tx0 + sub % SIDE * W, y0 = ty0 + sub / SIDE * W;
         // (a part of a tile may lie outside the image)
         const long long cap = SUB == 1 || (x0 < fc.width && y0 < fc.height) ? a.entries_cap : 0;
+        if constexpr (T == 64 && !LARGE) {
+            if (sub == SIDE * SIDE) {
+                whole_tile_lists(vs, a, w, fc, tx0, ty0, reinterpret_cast<float (*)[64][64]>(smem_raw));
+                finish(a, idx, t_start);
+                if (tid == 0) s_item[turn ^ 1] = next;
+                continue;
+            }
+        }
         if (list < 0 && tid < 4)
             s_range[tid] = a.offsets[fc.slot_base + (tid < 2 ? L_POINT : L_SMALL) * fc.ntiles + tile + (tid & 1)];
         // medium (tile pass) or large (large pass) particles into registers; never past
@@ -448,13 +502,15 @@ __global__ void __launch_bounds__(kTileThreads, kItemCtas) item_kernel(Views vs,
         const long long last = LARGE && T > 16 && a.cover ? item_full_start(a, fc, w) : w.end;
         const int n2 = mine ? (int)(min(last, cap) - lb2) : 0;
         float quad[2][2][3];
-        quad_list<W, (SUB > 1)>(a, a.entries + lb2, n2, x0, y0,
+        quad_list<W, (SIDE > 1)>(a, a.entries + lb2, n2, x0, y0,
                                 (unsigned)__cvta_generic_to_shared(smem_raw), quad);
 
         // points and small particles go through the shared tile, which reuses
         // the table space (the tables are dead once every warp is past here)
         long long lb0 = 0, le0 = 0, lb1 = 0, le1 = 0;
-        if (list < 0) {
+        if (SIDE > 1) {
+            // (see whole_tile_lists)
+        } else if (list < 0) {
             if (n2 <= 0) __syncthreads();   // s_range (the batches' barriers otherwise)
             lb0 = min(s_range[0], cap); le0 = min(s_range[1], cap);
             lb1 = min(s_range[2], cap); le1 = min(s_range[3], cap);
@@ -475,7 +531,7 @@ __global__ void __launch_bounds__(kTileThreads, kItemCtas) item_kernel(Views vs,
         // pass writes the tile: the large pass adds to what the tile pass left (687k
         // heavy-tailed particles on 3633 x 1145, one large item per tile: 0.112 ms with
         // atomic adds, 0.072 with plain ones)
-        const bool store = LARGE ? item_sole(w) : list < 0;
+        const bool store = LARGE ? item_sole(w) : list < 0 && SIDE == 1;
         const int onto = LARGE ? 1 : a.accumulate;
         float *image = a.images[view];
         const int64_t pitch = (int64_t)3 * fc.width;
@@ -539,13 +595,7 @@ __global__ void __launch_bounds__(kTileThreads, kItemCtas) item_kernel(Views vs,
                 for (int c = 0; c < 3; ++c) put_value(dst + c, v[c], store);
             }
         }
-        if (a.item_cycles) {
-            __syncthreads();
-            // (zeroed by the caller; the parts of a tile add up)
-            if (tid == 0)
-                atomicAdd(reinterpret_cast<unsigned long long *>(&a.item_cycles[idx]),
-                          (unsigned long long)(clock64() - t_start));
-        }
+        finish(a, idx, t_start);
         if (tid == 0) s_item[turn ^ 1] = next;
     }
 }
@@ -759,9 +809,7 @@ __global__ void __launch_bounds__(kTileThreads, kCoverCtas) cover_kernel(Views v
                 if (y0 + row < fc.height && x0 + x3 / 3 < fc.width)
                     put_value(image + (int64_t)3 * fc.width * (y0 + row) + 3 * x0 + x3, v[u], sole);
             }
-            if (a.item_cycles && tid == 0)
-                atomicAdd(reinterpret_cast<unsigned long long *>(&a.item_cycles[idx]),
-                          (unsigned long long)(clock64() - t_start));
+            finish(a, idx, t_start);
         }
     }
 }
