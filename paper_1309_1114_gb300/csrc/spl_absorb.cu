@@ -19,123 +19,96 @@ namespace spl {
 // C = C_1 + T_1 C_2 + T_1 T_2 C_3 ..., which is the same recurrence.
 // ---------------------------------------------------------------------------
 
-// Tables of one batch: swx[p][c] = (w_x, dx^2 B) as in the additive pass (for a
-// point: 1 in its column, 0 elsewhere, and no clip); srow[p][j] = (A w_y,
-// (r^2 - dy^2) B + 1) (a point: A in its row, 2 for the clip), or, where a
-// lane's rows go two at a time, per row pair (A w_a, A w_b, clip_a, clip_b);
-// ssrc[2p], ssrc[2p + 1] = (E / A) per channel, each value twice (0 when
-// A = 0), then A.  Thread (p, q) fills columns and rows (row pairs) q, q + 8, ... of
-// particle p and tests row band q.
-template <int T>
-__device__ __forceinline__ void absorb_tabulate(const FrameConst &fc, const float4 *st0,
-                                                const float4 *st1, const float2 *st2, int cnt,
-                                                int x0, int y0, float2 (*swx)[Shape<T>::WXS],
-                                                float2 (*srow)[Shape<T>::WXS], float4 *ssrc,
-                                                unsigned *band_mask, int tid) {
-    using S = Shape<T>;
-    const int p = tid >> 3, q = tid & 7;
-    // every lane runs to the end (band bits by ballot); entries of p >= cnt are
-    // written but never read
-    const bool valid = p < cnt;
-    const float4 r0 = st0[valid ? p : 0], r1 = st1[valid ? p : 0];
-    const float A = st2[valid ? p : 0].x, r2 = r1.x;
-    const bool point = r2 <= fc.r_sml2;
-    const int xi = unpack_xi(r0.x), yi = unpack_yi(r0.x);
+// Quarter-warps over 8 x 8 blocks, as in the additive pass (spl_tile.cu: blocks, bands,
+// parts of a tile), except that a pixel's particles must be taken in order.  The item's
+// list is cut into RANGES contiguous ranges; a batch holds 64 / RANGES particles of
+// each, and a quarter-warp takes its block's particles of its own range one after
+// the other: the two quarters of a block (and the four warps that share a pair of blocks at
+// W = 16) work on different ranges, whose (C, T) are composed at the end.
+//
+// What bounds it: issue and latency -- 24 packed operations per lane and step beside the
+// loads, and each pixel's T is a chain.  One particle per warp step over a 16 x 8 band, a
+// lane 2 x 2 pixels, records fetched between two barriers, took 9.48 ms on the
+// clustered 10M / 1024^2 frame (covered to 54 %; 8 x 8 blocks to 65 %); this takes
+// 8.15 ms.
+template <int W>
+struct Absorb {
+    static constexpr int P = 64;                   // particles per batch
+    // one particle's tables: W / 2 column pairs (w_a, w_b, dx_a^2 B, dx_b^2 B), W / 2 row
+    // pairs (A w_a, A w_b, rem_a, rem_b), then (E / A per channel, each value twice; A).  A point:
+    // 1 in its column and 0 elsewhere, A in its row, and no clip (0 and 2).  The odd
+    // number of 16-byte words puts neighbouring particles in different banks.
+    static constexpr int ROWS = 8 * W, SRC = 16 * W, BYTES = 16 * W + 48;
+    static constexpr int BL = W / 8, BANDS = BL * BL / 2, G = 8 / BANDS;   // as in Quad
+    static constexpr int RANGES = 2 * G, PER = P / RANGES;
+    static constexpr int kNone = P * BYTES;        // tables of a particle that changes nothing
+    static constexpr int kStage = kNone + BYTES;   // two batches of records and A
+    static constexpr int kStageBytes = P * 36;
+    static constexpr int kMask = kStage + 2 * kStageBytes;   // per block: the particles that reach it
+    static constexpr int kLists = kMask + 16 * 8;
+    static constexpr int LIST = 36;                // a block's particles of one range, padded
+    static constexpr int kSmem = kLists + 8 * 4 * LIST;
+    static_assert(kStage % 16 == 0 && kStageBytes % 16 == 0 && kMask % 16 == 0, "aligned");
+    static_assert(G == 1 || G * 16 * W * W <= kNone, "the tables hold the warps' partials");
+};
+constexpr int kAbsorbCtas = 3;      // per SM: 80 registers; with 4 (64, more spilling) 8.31 ms
+
+__device__ __forceinline__ void cp_async4(unsigned dst, const void *src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(src) : "memory");
+}
+__device__ __forceinline__ float lds1(unsigned a) {
+    float v;
+    asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(a));
+    return v;
+}
+
+// Tabulate the particle (r0, r1, A) into the block tab: thread q of its four fills column
+// pairs and row pairs q, q + 4, ....
+template <int W>
+__device__ __forceinline__ void absorb_tabulate(float4 r0, float4 r1, float A, bool point, int x0, int y0,
+                                                unsigned tab, int q) {
+    using Q = Absorb<W>;
     if (q == 0) {
-        // E / A per channel, each twice: the operand pairs of the packed FMAs
         const float inv = A > 0.f ? 1.f / A : 0.f;
         const float e0 = r1.y * inv, e1 = r1.z * inv, e2 = r1.w * inv;
-        ssrc[2 * p] = make_float4(e0, e0, e1, e1);
-        ssrc[2 * p + 1] = make_float4(e2, e2, A, 0.f);
+        sts2x2(tab + Q::SRC, pack2(e0, e0), pack2(e1, e1));
+        sts2x2(tab + Q::SRC + 16, pack2(e2, e2), pack2(A, 0.f));
     }
-    // row table: per row (A w_y, clip term), or per row pair (A w_a, A w_b,
-    // clip_a, clip_b) when rows go two at a time
-    float4 *srow4 = reinterpret_cast<float4 *>(&srow[0][0]);
-    int ilo, ihi, jlo, jhi;
-    float r = 0.f, xh = 0.f, yh = 0.f;
-    if (point) {
-        ilo = ihi = xi - x0;
-        jlo = jhi = yi - y0;
+    const int cx = unpack_xi(r0.x) - x0, cy = unpack_yi(r0.x) - y0;   // the point's pixel
+    const float B = __fdividef(1048576.f, r1.x);
+    const f32x2 nkq = pack2(-r0.w, -r0.w), B2 = pack2(B, B), AA = pack2(A, A);
+    const float xf = (float)(2 * q - cx), yf = (float)(2 * q - cy);
+    const f32x2 x2 = pack2(xf, xf + 1.f), y2 = pack2(yf, yf + 1.f);
+    const f32x2 xh = pack2(0.5f - r0.y, 0.5f - r0.y), yh = pack2(0.5f - r0.z, 0.5f - r0.z);
+    const f32x2 rr = pack2(r1.x, r1.x), one = pack2(1.f, 1.f), mone = pack2(-1.f, -1.f);
 #pragma unroll
-        for (int u = 0; u < S::PER; ++u) {
-            const int k = q + 8 * u;
-            swx[p][k] = make_float2(x0 + k == xi ? 1.f : 0.f, 0.f);
-            if constexpr (!S::PAIRED) srow[p][k] = make_float2(y0 + k == yi ? A : 0.f, 2.f);
+    for (int u = 0; u < W / 8; ++u) {
+        const unsigned at = tab + 16 * q + 64 * u;
+        if (point) {
+            const int k = 2 * q + 8 * u;
+            sts2x2(at, pack2(k == cx ? 1.f : 0.f, k + 1 == cx ? 1.f : 0.f), 0ull);
+            sts2x2(at + Q::ROWS, pack2(k == cy ? A : 0.f, k + 1 == cy ? A : 0.f), pack2(2.f, 2.f));
+            continue;
         }
-        if constexpr (S::PAIRED) {
-#pragma unroll
-            for (int u = 0; u < S::PER / 2; ++u) {
-                const int m = q + 8 * u;
-                srow4[p * (T / 2) + m] = make_float4(y0 + 2 * m == yi ? A : 0.f,
-                                                     y0 + 2 * m + 1 == yi ? A : 0.f, 2.f, 2.f);
-            }
-        }
-    } else {
-        const float kq = r0.w, B = __fdividef(1048576.f, r2);
-        xh = 0.5f - r0.y;
-        yh = 0.5f - r0.z;
-        r = r2 * rsqrtf(r2) + 1e-3f;   // approximate: far inside the margin
-        ilo = xi - x0 + (int)ceilf(fmaxf(r0.y - 0.5f - r, -1e6f));
-        ihi = xi - x0 + (int)floorf(fminf(r0.y - 0.5f + r, 1e6f));
-        jlo = yi - y0 + (int)ceilf(fmaxf(r0.z - 0.5f - r, -1e6f));
-        jhi = yi - y0 + (int)floorf(fminf(r0.z - 0.5f + r, 1e6f));
-#pragma unroll
-        for (int u = 0; u < S::PER; ++u) {
-            const int k = q + 8 * u;
-            const float dx = (float)(x0 + k - xi) + xh;
-            const float dx2 = dx * dx;
-            swx[p][k] = make_float2(ex2_neg(kq * dx2), dx2 * B);
-            if constexpr (!S::PAIRED) {
-                const float dy = (float)(y0 + k - yi) + yh;
-                const float dy2 = dy * dy;
-                srow[p][k] = make_float2(A * ex2_neg(kq * dy2), fmaf(r2 - dy2, B, 1.f));
-            }
-        }
-        if constexpr (S::PAIRED) {
-#pragma unroll
-            for (int u = 0; u < S::PER / 2; ++u) {
-                const int m = q + 8 * u;
-                const float dya = (float)(y0 + 2 * m - yi) + yh, dyb = dya + 1.f;
-                const float a2 = dya * dya, b2 = dyb * dyb;
-                srow4[p * (T / 2) + m] =
-                    make_float4(A * ex2_neg(kq * a2), A * ex2_neg(kq * b2), fmaf(r2 - a2, B, 1.f),
-                                fmaf(r2 - b2, B, 1.f));
-            }
-        }
-    }
-    // band q: box overlap, and for a disc its reach to the band's nearest pixel
-    // centre (as in the additive pass); a warp's four particles by one ballot
-    const int bx0 = (q % S::NBX) * S::BW, by0 = (q / S::NBX) * S::BH;
-    const int bx1 = bx0 + S::BW - 1, by1 = by0 + S::BH - 1;
-    bool hit = valid && jhi >= by0 && jlo <= by1 && ihi >= bx0 && ilo <= bx1;
-    if (!point) {
-        const float ax = (float)(x0 + bx0 - xi) + xh, ay = (float)(y0 + by0 - yi) + yh;
-        const float nx = fmaxf(ax, fminf(0.f, ax + (float)(S::BW - 1)));
-        const float ny = fmaxf(ay, fminf(0.f, ay + (float)(S::BH - 1)));
-        hit = hit && nx * nx + ny * ny <= r * r;
-    }
-    const unsigned hb = __ballot_sync(0xffffffffu, hit);
-    const int lane = tid & 31;
-    if (lane < 8) {
-        const unsigned nib = ((hb >> lane) & 1u) | (((hb >> (lane + 8)) & 1u) << 1) |
-                             (((hb >> (lane + 16)) & 1u) << 2) | (((hb >> (lane + 24)) & 1u) << 3);
-        if (nib) atomicOr(&band_mask[lane], nib << (4 * (tid >> 5)));
+        const f32x2 dx = add2(add2(x2, pack2(8.f * u, 8.f * u)), xh);
+        const f32x2 dy = add2(add2(y2, pack2(8.f * u, 8.f * u)), yh);
+        const f32x2 dx2 = mul2(dx, dx), dy2 = mul2(dy, dy);
+        float ta, tb, wa, wb;
+        unpack2(mul2(dx2, nkq), ta, tb);
+        asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(wa) : "f"(ta));
+        asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(wb) : "f"(tb));
+        sts2x2(at, pack2(wa, wb), mul2(dx2, B2));
+        unpack2(mul2(dy2, nkq), ta, tb);
+        asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(wa) : "f"(ta));
+        asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(wb) : "f"(tb));
+        sts2x2(at + Q::ROWS, mul2(AA, pack2(wa, wb)), fma2v(fma2v(dy2, mone, rr), B2, one));
     }
 }
 
-// 1 - exp(-tau) for tau >= 0 with small relative error everywhere: below
-// 1/16 the Taylor series to tau^5 (truncation < tau^5/720 relative, < 2e-9),
+// 1 - exp(-tau) for tau >= 0, two values at once, with small relative error everywhere:
+// below 1/16 the Taylor series to tau^5 (truncation < tau^5/720 relative, < 2e-9),
 // above it one minus the hardware exp2 (relative error there < 16 * 2^-22).
 // Computing 1 - exp(-tau) directly would lose all digits of a small tau.
-__device__ __forceinline__ float one_minus_exp_neg(float tau) {
-    const float series =
-        tau * fmaf(tau, fmaf(tau, fmaf(tau, fmaf(tau, 1.f / 120.f, -1.f / 24.f), 1.f / 6.f), -0.5f), 1.f);
-    return tau < 0.0625f ? series : 1.f - ex2_neg(1.4426950408889634f * tau);
-}
-
-// The same for two values at once: the series and one minus the hardware exp2
-// as packed FP32x2 operations (each half rounded as the scalar instruction, so
-// the results equal one_minus_exp_neg's bit for bit).
 __device__ __forceinline__ f32x2 one_minus_exp_neg2(f32x2 tau) {
     const f32x2 c5 = pack2(1.f / 120.f, 1.f / 120.f), c4 = pack2(-1.f / 24.f, -1.f / 24.f);
     const f32x2 c3 = pack2(1.f / 6.f, 1.f / 6.f), c2 = pack2(-0.5f, -0.5f);
@@ -161,8 +134,8 @@ __device__ __forceinline__ f32x2 one_minus_exp_neg2(f32x2 tau) {
 // The same where tau <= 1, two values at once: tau times the degree-5 Chebyshev
 // interpolant of (1 - exp(-tau)) / tau on [0, 1] (relative error 9.4e-8; with FP32
 // rounding at most 2.0e-7, 6.7e-8 rms).  A particle with 0 <= A <= 1 never exceeds it,
-// since its weights are at most 1, so that the choice is the same for the whole
-// warp; per pixel pair it saves the hardware exp2s, the branch's two compares and
+// since its weights are at most 1, so that the choice is made once per warp step;
+// per pixel pair it saves the hardware exp2s, the branch's two compares and
 // selects and two packed operations.
 __device__ __forceinline__ f32x2 one_minus_exp_neg2_unit(f32x2 tau) {
     f32x2 sr = fma2v(tau, pack2(-0.000912545391f, -0.000912545391f), pack2(0.00783736380f, 0.00783736380f));
@@ -173,190 +146,237 @@ __device__ __forceinline__ f32x2 one_minus_exp_neg2_unit(f32x2 tau) {
     return mul2(tau, sr);
 }
 
-template <int T>
-__host__ __device__ constexpr size_t absorb_smem_bytes() {
-    using S = Shape<T>;
-    return (sizeof(float2) * 2 * S::WXS + 2 * sizeof(float4)) * S::P +   // swx, srow, ssrc
-           (2 * sizeof(float4) + sizeof(float2)) * S::P;              // staged records
+// The step of one particle for a lane's 4 x 2 pixels, with either form of 1 - exp(-tau).
+template <bool UNIT>
+__device__ __forceinline__ void absorb_step(f32x2 (&tr)[4], f32x2 (&col)[4][3], const float (&wx)[4],
+                                            const float (&dxb)[4], f32x2 aw, float rem_a, float rem_b,
+                                            f32x2 s0, f32x2 s1, f32x2 s2) {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const f32x2 clip = pack2(__saturatef(rem_a - dxb[k]), __saturatef(rem_b - dxb[k]));
+        const f32x2 tau = mul2(mul2(pack2(wx[k], wx[k]), clip), aw);
+        const f32x2 f = mul2(tr[k], UNIT ? one_minus_exp_neg2_unit(tau) : one_minus_exp_neg2(tau));
+        fma2(col[k][0], f, s0);
+        fma2(col[k][1], f, s1);
+        fma2(col[k][2], f, s2);
+        tr[k] = fma2v(f, pack2(-1.f, -1.f), tr[k]);
+    }
 }
 
-// CTAs per SM.  The pass is latency-bound (each pixel's transmittance is a
-// chain across its list), so occupancy pays: at T = 32, 2 -> 4 -> 6 CTAs per
-// SM (106 -> 62 -> 40 registers, 8 bytes spilled at 40) took the clustered
-// 10M / 1024^2 pass from 15.2 to 11.3 to 10.7 ms.  At T = 64 a lane's 16
-// pixels need the registers of 2 CTAs per SM; at T = 16, 5 fit without spills.
-template <int T>
-constexpr int absorb_ctas() { return T == 64 ? 2 : (T == 32 ? 6 : 5); }
+// (C, T) of what lies in front, then of what lies behind it.
+__device__ __forceinline__ float4 compose(float4 front, float4 back) {
+    return make_float4(fmaf(front.w, back.x, front.x), fmaf(front.w, back.y, front.y),
+                       fmaf(front.w, back.z, front.z), front.w * back.w);
+}
 
 template <int T>
-__global__ void __launch_bounds__(kTileThreads, absorb_ctas<T>()) absorb_kernel(Views vs, TileArgs a) {
-    using S = Shape<T>;
+__global__ void __launch_bounds__(kTileThreads, kAbsorbCtas) absorb_kernel(Views vs, TileArgs a) {
+    constexpr int W = T == 16 ? 16 : 32, SIDE = T / W, SUB = SIDE * SIDE;
+    using Q = Absorb<W>;
+    constexpr int P = Q::P, BL = Q::BL;
     extern __shared__ float4 smem_raw[];
-    float2 (*swx)[S::WXS] = reinterpret_cast<float2 (*)[S::WXS]>(smem_raw);
-    float2 (*srow)[S::WXS] = swx + S::P;
-    float4 *ssrc = reinterpret_cast<float4 *>(srow + S::P);   // two per particle
-    float4 *st0 = ssrc + 2 * S::P;
-    float4 *st1 = st0 + S::P;
-    float2 *st2 = reinterpret_cast<float2 *>(st1 + S::P);
-    __shared__ unsigned band_mask[kTileThreads / 32];
-    __shared__ int s_item;
-    __shared__ FrameConst sfc;
+    __shared__ int s_item[2];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int n_items = min(a.st->item_totals[0], a.items_cap);
-    for (;;) {
+    const int n_work = min(a.st->item_totals[0], a.items_cap) * SUB;
+    const unsigned smem = (unsigned)__cvta_generic_to_shared(smem_raw);
+    if (tid < Q::BYTES / 16) smem_raw[Q::kNone / 16 + tid] = make_float4(0.f, 0.f, 0.f, 0.f);
+    const int band = warp % Q::BANDS, group = warp / Q::BANDS;
+    const int brow = band / (BL / 2), bcol = band % (BL / 2) * 2;     // left block of the pair
+    const unsigned lt = (1u << lane) - 1u;
+    const int quarter = lane >> 3, side = quarter >> 1, cg = lane & 1, rg = (lane >> 1) & 3;
+    const bool behind = quarter & 1;               // this quarter's range of the pair 2 group, 2 group + 1
+    const unsigned col_at = smem + (unsigned)((bcol + side) * 8 + 4 * cg) * 8u;
+    const unsigned row_at = smem + Q::ROWS + (unsigned)(brow * 4 + rg) * 16u;
+    const unsigned lists = smem + Q::kLists + (unsigned)(4 * warp) * Q::LIST;
+    // threads 2p, 2p + 1 copy the halves of staged record p, thread 128 + p its A
+    const int sp = tid < 2 * P ? tid >> 1 : tid - 2 * P;
+    const bool copies = tid < 3 * P;
+    const unsigned stage_at = smem + Q::kStage +
+                              (tid < 2 * P ? (unsigned)(tid & 1) * (P * 16) + (unsigned)sp * 16u
+                                           : (unsigned)(P * 32) + (unsigned)sp * 4u);
+    int next = 0;
+    if (tid == 0) s_item[0] = atomicAdd(&a.st->item_counter[0], 1);
+    for (int turn = 0;; turn ^= 1) {
         __syncthreads();
-        if (tid == 0) s_item = atomicAdd(&a.st->item_counter[0], 1);
-        __syncthreads();
-        const int it = s_item;
-        if (it >= n_items) break;
-        const int idx = a.order ? a.order[it] : it;
+        const int it = s_item[turn];
+        if (it >= n_work) break;
+        if (tid == 0) next = atomicAdd(&a.st->item_counter[0], 1);
+        const int idx = a.order ? a.order[it / SUB] : it / SUB, sub = it % SUB;
         const WorkItem w = a.items[idx];
         const int view = item_view(w), list = item_list(w);
-        {
-            const int words = (int)(sizeof(FrameConst) / sizeof(int));
-            if (tid < words)
-                reinterpret_cast<int *>(&sfc)[tid] = reinterpret_cast<const int *>(vs.fcs + view)[tid];
+        const FrameConst &fc = vs.fcs[view];
+        const int tile = w.tile - fc.tile_base, width = fc.width, height = fc.height;
+        const int x0 = (tile % fc.ntx) * T + sub % SIDE * W, y0 = (tile / fc.ntx) * T + sub / SIDE * W;
+        const float r_sml2 = fc.r_sml2;
+        const int n_ent = SUB > 1 && (x0 >= width || y0 >= height) ? 0 : (int)(w.end - w.start);
+        const unsigned *ent = a.entries + w.start;
+        // the staged slot's range and place in it
+        const int range = sp / Q::PER;
+        const int e0 = (int)((long long)n_ent * range / Q::RANGES) + sp % Q::PER;
+        const int e1 = (int)((long long)n_ent * (range + 1) / Q::RANGES);
+        const int batches = ((n_ent + Q::RANGES - 1) / Q::RANGES + Q::PER - 1) / Q::PER;
+        auto stage_copy = [&](unsigned id, unsigned buf) {
+            if (tid < 2 * P)
+                cp_async16(stage_at + buf * Q::kStageBytes,
+                           reinterpret_cast<const char *>(a.recs + id) + (tid & 1) * 16);
+            else
+                cp_async4(stage_at + buf * Q::kStageBytes, &a.rec2[id].x);
+        };
+        f32x2 tr[4], col[4][3];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            tr[k] = pack2(1.f, 1.f);
+            col[k][0] = col[k][1] = col[k][2] = 0ull;
         }
-        __syncthreads();
-        const FrameConst &fc = sfc;
-        const int tile = w.tile - fc.tile_base;
-        const int x0 = (tile % fc.ntx) * T, y0 = (tile / fc.ntx) * T;
-        long long lb = w.start, le = w.end;
-        if (list < 0) {
-            lb = a.offsets[fc.slot_base + L_MEDIUM * fc.ntiles + tile];
-            le = a.offsets[fc.slot_base + L_MEDIUM * fc.ntiles + tile + 1];
-        }
-        const int col = (warp % S::NBX) * S::BW + (lane % S::LW) * S::CMUL;
-        const int row0 = (warp / S::NBX) * S::BH + (lane / S::LW) * S::RPL;
-        // (T, C) per pixel in registers: scalar, or two rows per FP32x2 pair
-        constexpr int RP = S::PAIRED ? S::RPL / 2 : 1;
-        float Tr[S::RPL][S::CPL], C[S::RPL][S::CPL][3];
-        f32x2 Tr2[RP][S::CPL], C2[RP][S::CPL][3];
-        if constexpr (S::PAIRED) {
-#pragma unroll
-            for (int m = 0; m < RP; ++m)
-#pragma unroll
-                for (int k = 0; k < S::CPL; ++k) {
-                    Tr2[m][k] = pack2(1.f, 1.f);
-                    C2[m][k][0] = C2[m][k][1] = C2[m][k][2] = 0ull;
-                }
-        } else {
-#pragma unroll
-            for (int q = 0; q < S::RPL; ++q)
-#pragma unroll
-                for (int k = 0; k < S::CPL; ++k) {
-                    Tr[q][k] = 1.f;
-                    C[q][k][0] = C[q][k][1] = C[q][k][2] = 0.f;
-                }
+        unsigned id = 0, buf = 0;
+        if (copies && e0 < e1) {
+            stage_copy(ent[e0], 0u);
+            if (e0 + Q::PER < e1) id = ent[e0 + Q::PER];
         }
 #pragma unroll 1
-        for (long long base = lb; base < le; base += S::P) {
-            const int cnt = (int)(le - base < S::P ? le - base : S::P);
-            if (tid < cnt) {
-                const unsigned id = a.entries[base + tid];
-                const Rec rc = a.recs[id];
-                st0[tid] = rc.r0;
-                st1[tid] = rc.r1;
-                st2[tid] = a.rec2[id];
+        for (int b = 0; b < batches; ++b) {
+            const unsigned st = smem + Q::kStage + buf * Q::kStageBytes;
+            cp_async_wait();
+            __syncthreads();
+            const int en = e0 + (b + 1) * Q::PER;
+            if (copies && en < e1) {
+                stage_copy(id, buf ^ 1u);
+                if (en + Q::PER < e1) id = ent[en + Q::PER];
             }
-            if (tid < kTileThreads / 32) band_mask[tid] = 0u;
-            __syncthreads();
-            absorb_tabulate<T>(fc, st0, st1, st2, cnt, x0, y0, swx, srow, ssrc, band_mask, tid);
-            __syncthreads();
-            // this warp's band, particles front to back (increasing list position)
-            unsigned mask = band_mask[warp];
-            while (mask) {
-                const int p = __ffs(mask) - 1;
-                mask &= mask - 1u;
-                float wx[S::CPL], dxb[S::CPL];
-                if constexpr (S::CSTEP == 1 && S::CPL == 2) {
-                    // two adjacent columns in one 16-byte load (col is even)
-                    const float4 v = *reinterpret_cast<const float4 *>(&swx[p][col]);
-                    wx[0] = v.x; dxb[0] = v.y; wx[1] = v.z; dxb[1] = v.w;
-                } else {
+            {
+                const int p = tid >> 2, q = tid & 3, rp = p / Q::PER;
+                bool valid = (int)((long long)n_ent * rp / Q::RANGES) + p % Q::PER + b * Q::PER <
+                             (int)((long long)n_ent * (rp + 1) / Q::RANGES);
+                const float4 r0 = lds4(st + p * 16), r1 = lds4(st + P * 16 + p * 16);
+                const float A = lds1(st + P * 32 + p * 4);
+                // the blocks in row q of blocks that the particle reaches (a point: its
+                // pixel's; a disc, with a margin, their pixel centres), as in the additive pass
+                const bool point = r1.x <= r_sml2;
+                const int cx = unpack_xi(r0.x) - x0, cy = unpack_yi(r0.x) - y0;
+                const float r = r1.x * rsqrtf(r1.x) + 1e-3f;      // approximate: far inside the margin
+                const float ax = (float)-cx + (0.5f - r0.y), ay = (float)(8 * q - cy) + (0.5f - r0.z);
+                const float ny = fmaxf(ay, fminf(0.f, ay + 7.f)), room = r * r - ny * ny;
+                unsigned bits = 0, any = 0;
 #pragma unroll
-                    for (int k = 0; k < S::CPL; ++k) {
-                        const float2 v = swx[p][col + S::CSTEP * k];
-                        wx[k] = v.x;
-                        dxb[k] = v.y;
-                    }
+                for (int u = 0; u < BL; ++u) {
+                    const float nx = fmaxf(ax + (float)(8 * u), fminf(0.f, ax + (float)(8 * u + 7)));
+                    const bool hit = point ? cx >> 3 == u && cy >> 3 == q : nx * nx <= room;
+                    const unsigned h = __ballot_sync(0xffffffffu, valid && q < BL && hit);
+                    if ((lane & (BL - 1)) == u) bits = h;
+                    any |= h;
                 }
-                if constexpr (S::PAIRED) {
-                    // per row pair: (A w_a, A w_b) and the two clip terms; E / A
-                    // per channel as duplicated pairs
-                    const ulonglong2 *sv = reinterpret_cast<const ulonglong2 *>(ssrc) + 2 * p;
-                    const ulonglong2 s01 = sv[0], s2x = sv[1];
-                    const ulonglong2 *rp =
-                        reinterpret_cast<const ulonglong2 *>(&srow[0][0]) + p * (T / 2) + row0 / 2;
-                    float A, unused;
-                    unpack2(s2x.y, A, unused);
-                    const bool thin = A >= 0.f && A <= 1.f;
-#pragma unroll
-                    for (int m = 0; m < RP; ++m) {
-                        const ulonglong2 rv = rp[m];
-                        float ca, cb;
-                        unpack2(rv.y, ca, cb);
-#pragma unroll
-                        for (int k = 0; k < S::CPL; ++k) {
-                            const f32x2 clip =
-                                pack2(__saturatef(ca - dxb[k]), __saturatef(cb - dxb[k]));
-                            const f32x2 tau = mul2(mul2(pack2(wx[k], wx[k]), clip), rv.x);
-                            const f32x2 f = mul2(Tr2[m][k], thin ? one_minus_exp_neg2_unit(tau) : one_minus_exp_neg2(tau));
-                            fma2(C2[m][k][0], f, s01.x);
-                            fma2(C2[m][k][1], f, s01.y);
-                            fma2(C2[m][k][2], f, s2x.x);
-                            Tr2[m][k] = fma2v(f, pack2(-1.f, -1.f), Tr2[m][k]);
-                        }
-                    }
-                } else {
-                    const float4 src = ssrc[2 * p];
-                    const float src2 = ssrc[2 * p + 1].x;
-#pragma unroll
-                    for (int q = 0; q < S::RPL; ++q) {
-                        const float2 rv = srow[p][row0 + q];
-#pragma unroll
-                        for (int k = 0; k < S::CPL; ++k) {
-                            const float tau = wx[k] * __saturatef(rv.y - dxb[k]) * rv.x;
-                            const float g = one_minus_exp_neg(tau);
-                            const float f = Tr[q][k] * g;                 // T (1 - e^-tau)
-                            C[q][k][0] = fmaf(f, src.x, C[q][k][0]);
-                            C[q][k][1] = fmaf(f, src.z, C[q][k][1]);
-                            C[q][k][2] = fmaf(f, src2, C[q][k][2]);
-                            Tr[q][k] -= f;                                // T e^-tau
-                        }
-                    }
+                if (lane < BL * BL) {
+                    const unsigned m = every_fourth(bits >> (lane / BL));
+                    asm volatile("st.shared.u8 [%0], %1;" ::"r"(smem + Q::kMask + 8 * lane + warp), "r"(m)
+                                 : "memory");
                 }
+                if (SUB > 1) valid = (any >> (lane & ~3)) & 0xfu;
+                if (valid) absorb_tabulate<W>(r0, r1, A, point, x0, y0, smem + p * Q::BYTES, q);
             }
             __syncthreads();
+            // per quarter: its block's particles of its range, in order, padded to the
+            // longest of the warp's four
+            const unsigned masks = smem + Q::kMask + 8u * (unsigned)(brow * BL + bcol);
+            uint4 m;
+            if (Q::G == 1) {
+                m = ldsu4(masks);
+            } else {
+                const unsigned l = lds_u16(masks + 2 * group), r = lds_u16(masks + 8 + 2 * group);
+                m = make_uint4(l & 0xffu, l >> 8, r & 0xffu, r >> 8);
+            }
+            const int first = 2 * group * Q::PER + lane;
+            const int n0 = __popc(m.x), n1 = __popc(m.y), n2 = __popc(m.z), n3 = __popc(m.w);
+            const int n = max(max(n0, n1), max(n2, n3));
+            if (n0 + lane <= n) sts_u8(lists + n0 + lane, P);
+            if (n1 + lane <= n) sts_u8(lists + Q::LIST + n1 + lane, P);
+            if (n2 + lane <= n) sts_u8(lists + 2 * Q::LIST + n2 + lane, P);
+            if (n3 + lane <= n) sts_u8(lists + 3 * Q::LIST + n3 + lane, P);
+            if ((m.x >> lane) & 1u) sts_u8(lists + __popc(m.x & lt), first);
+            if ((m.y >> lane) & 1u) sts_u8(lists + Q::LIST + __popc(m.y & lt), first + Q::PER);
+            if ((m.z >> lane) & 1u) sts_u8(lists + 2 * Q::LIST + __popc(m.z & lt), first);
+            if ((m.w >> lane) & 1u) sts_u8(lists + 3 * Q::LIST + __popc(m.w & lt), first + Q::PER);
+            __syncwarp();
+            unsigned at = lists + (unsigned)quarter * Q::LIST;
+            unsigned off = lds_u8(at);
+#pragma unroll 1
+            for (int i = 0; i < n; ++i) {
+                const unsigned tab = off * Q::BYTES;
+                ++at;
+                off = lds_u8(at);
+                const float4 c0 = lds4(col_at + tab), c1 = lds4(col_at + tab + 16);
+                f32x2 aw, rem, s0, s1, s2, av;
+                lds2x2(row_at + tab, aw, rem);
+                lds2x2(smem + Q::SRC + tab, s0, s1);
+                lds2x2(smem + Q::SRC + 16 + tab, s2, av);
+                const float wx[4] = {c0.x, c0.y, c1.x, c1.y}, dxb[4] = {c0.z, c0.w, c1.z, c1.w};
+                float rem_a, rem_b, A, unused;
+                unpack2(rem, rem_a, rem_b);
+                unpack2(av, A, unused);
+                if (__all_sync(0xffffffffu, A >= 0.f && A <= 1.f))
+                    absorb_step<true>(tr, col, wx, dxb, aw, rem_a, rem_b, s0, s1, s2);
+                else
+                    absorb_step<false>(tr, col, wx, dxb, aw, rem_a, rem_b, s0, s1, s2);
+            }
+            buf ^= 1u;
+        }
+        // the quarters of a block compose their ranges: the front one keeps columns 0 and 1,
+        // the one behind 2 and 3
+        float4 px[2][2];
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            float mine[2][4], theirs[2][4];
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                const f32x2 a2 = c < 3 ? col[k][c < 3 ? c : 0] : tr[k], b2 = c < 3 ? col[k + 2][c < 3 ? c : 0] : tr[k + 2];
+                float a0, a1, b0, b1;
+                unpack2(a2, a0, a1);
+                unpack2(b2, b0, b1);
+                mine[0][c] = behind ? b0 : a0;
+                mine[1][c] = behind ? b1 : a1;
+                theirs[0][c] = __shfl_xor_sync(0xffffffffu, behind ? a0 : b0, 8);
+                theirs[1][c] = __shfl_xor_sync(0xffffffffu, behind ? a1 : b1, 8);
+            }
+#pragma unroll
+            for (int y = 0; y < 2; ++y) {
+                const float4 u = make_float4(mine[y][0], mine[y][1], mine[y][2], mine[y][3]);
+                const float4 v = make_float4(theirs[y][0], theirs[y][1], theirs[y][2], theirs[y][3]);
+                px[k][y] = behind ? compose(v, u) : compose(u, v);
+            }
         }
         float *image = a.images[view];
-#pragma unroll
-        for (int q = 0; q < S::RPL; ++q) {
-            const int row = row0 + q;
-#pragma unroll
-            for (int k = 0; k < S::CPL; ++k) {
-                float c0, c1, c2, tr;
-                if constexpr (S::PAIRED) {
-                    float lo, hi;
-                    unpack2(C2[q >> 1][k][0], lo, hi); c0 = (q & 1) ? hi : lo;
-                    unpack2(C2[q >> 1][k][1], lo, hi); c1 = (q & 1) ? hi : lo;
-                    unpack2(C2[q >> 1][k][2], lo, hi); c2 = (q & 1) ? hi : lo;
-                    unpack2(Tr2[q >> 1][k], lo, hi); tr = (q & 1) ? hi : lo;
-                } else {
-                    c0 = C[q][k][0]; c1 = C[q][k][1]; c2 = C[q][k][2]; tr = Tr[q][k];
-                }
-                const int cx = col + S::CSTEP * k;
-                if (y0 + row >= fc.height || x0 + cx >= fc.width) continue;
-                if (list < 0) {
-                    float *dst = image + 3 * ((int64_t)(y0 + row) * fc.width + x0 + cx);
-                    dst[0] = c0;
-                    dst[1] = c1;
-                    dst[2] = c2;
-                } else {
-                    a.partial[(size_t)idx * (T * T) + row * T + cx] = make_float4(c0, c1, c2, tr);
-                }
+        auto put = [&](int row, int cx, float4 v) {
+            if (y0 + row >= height || x0 + cx >= width) return;
+            if (list < 0) {
+                float *dst = image + 3 * ((int64_t)(y0 + row) * width + x0 + cx);
+                dst[0] = v.x;
+                dst[1] = v.y;
+                dst[2] = v.z;
+            } else {
+                a.partial[(size_t)idx * (T * T) + (sub / SIDE * W + row) * T + sub % SIDE * W + cx] = v;
             }
+        };
+        const int row = brow * 8 + rg * 2, cx = (bcol + side) * 8 + cg * 4 + (behind ? 2 : 0);
+        if constexpr (Q::G == 1) {
+#pragma unroll
+            for (int k = 0; k < 2; ++k)
+#pragma unroll
+                for (int y = 0; y < 2; ++y) put(row + y, cx + k, px[k][y]);
+        } else {
+            // the warps that share a pair of blocks, in the order of their ranges
+            float4 (*part)[W * W] = reinterpret_cast<float4 (*)[W * W]>(smem_raw);
+            __syncthreads();
+#pragma unroll
+            for (int k = 0; k < 2; ++k)
+#pragma unroll
+                for (int y = 0; y < 2; ++y) part[group][(row + y) * W + cx + k] = px[k][y];
+            __syncthreads();
+            static_assert(Q::G == 1 || W * W == kTileThreads, "one pixel per thread");
+            float4 v = part[0][tid];
+#pragma unroll
+            for (int g = 1; g < Q::G; ++g) v = compose(v, part[g][tid]);
+            put(tid / W, tid % W, v);
         }
+        if (tid == 0) s_item[turn ^ 1] = next;
     }
 }
 
@@ -366,7 +386,7 @@ __global__ void __launch_bounds__(kTileThreads, absorb_ctas<T>()) absorb_kernel(
 // Bound by the partials' traffic (16 B per pixel and item): a crowded tile has
 // hundreds of items, and one thread per pixel running through all of them in four
 // passes of a single CTA per tile was a chain of loads (597 us for the clustered
-// 10M / 1024^2 frame; now COMBINE_US).
+// 10M / 1024^2 frame; now 94 us).
 template <int T>
 __global__ void __launch_bounds__(256) absorb_combine_kernel(Views vs, const int *item_offsets,
                                                              const float4 *partial,
@@ -416,8 +436,9 @@ __global__ void __launch_bounds__(256) absorb_combine_kernel(Views vs, const int
 template <int T>
 static void launch_absorb_t(const Views &vs, const TileArgs &a, const int *item_offsets, int sms,
                             cudaStream_t s) {
-    constexpr size_t bytes = absorb_smem_bytes<T>();
-    absorb_kernel<T><<<sms * absorb_ctas<T>(), kTileThreads, bytes, s>>>(vs, a);
+    constexpr size_t bytes = Absorb<(T == 16 ? 16 : 32)>::kSmem;
+    cudaFuncSetAttribute(absorb_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    absorb_kernel<T><<<sms * kAbsorbCtas, kTileThreads, bytes, s>>>(vs, a);
     ++g_launches;
     const long long units = (long long)vs.total_tiles * (T * T / 32);
     const int grid = (int)(units < sms * 8 ? units : sms * 8);

@@ -204,14 +204,6 @@ __device__ __forceinline__ void quad_tabulate(float4 r0, float4 r1, int x0, int 
     }
 }
 
-// Bits 0, 4, ..., 28 of v gathered into the low byte.
-__device__ __forceinline__ unsigned every_fourth(unsigned v) {
-    v &= 0x11111111u;
-    v = (v | (v >> 3)) & 0x03030303u;
-    v = (v | (v >> 6)) & 0x000f000fu;
-    return (v | (v >> 12)) & 0xffu;
-}
-
 // The n_ent list entries at ent into this lane's pixels: v[k][y][c] = channel c of row
 // (2 rg + y), column (4 cg + 2 (quarter & 1) + k) of the lane's block.  FILTER: some of the
 // list's particles miss these pixels altogether.

@@ -1,33 +1,17 @@
 // spl_tile.cuh -- shared-memory access by address for the additive passes
-// (spl_tile.cu), and the band geometry of the general absorption pass
-// (spl_absorb.cu).
+// (spl_tile.cu) and the general absorption pass (spl_absorb.cu).
 #pragma once
 #include "spl_geom.cuh"
 
 namespace spl {
 
-template <int T>
-struct Shape {
-    // A tile is cut into 8 row bands, one per warp: BW columns x BH rows.
-    static constexpr int BW = T == 64 ? 64 : 16;
-    static constexpr int BH = T * T / (8 * BW);
-    static constexpr int NBX = T / BW;             // bands across the tile
-    // lanes along a band row: 8 for T = 32, so that a lane's two columns
-    // share each row-pair load and the column table is read 16 bytes at a time
-    static constexpr int LW = T == 32 ? 8 : (BW < 32 ? BW : 32);
-    // a lane's columns: col + CSTEP k, k < CPL, col = band column + CMUL * (lane % LW)
-    static constexpr int CSTEP = T == 32 ? 1 : 32;
-    static constexpr int CMUL = T == 32 ? 2 : 1;
-    static constexpr int G = 32 / LW;              // lane groups (rows split between them)
-    static constexpr int CPL = BW / LW;            // columns per lane
-    static constexpr int RPL = BH / G;             // rows per lane
-    static constexpr int P = 32;                   // particles per tabulated batch
-    static constexpr int PER = T / 8;              // table columns (and rows) per thread
-    static constexpr bool PAIRED = RPL % 2 == 0;   // rows two at a time (FP32x2)
-    // row stride of the column table: 8 entries of padding put the two
-    // particles that a half-warp's 64-bit stores reach in different banks
-    static constexpr int WXS = T + 8;
-};
+// Bits 0, 4, ..., 28 of v gathered into the low byte.
+__device__ __forceinline__ unsigned every_fourth(unsigned v) {
+    v &= 0x11111111u;
+    v = (v | (v >> 3)) & 0x03030303u;
+    v = (v | (v >> 6)) & 0x000f000fu;
+    return (v | (v >> 12)) & 0xffu;
+}
 
 // Shared memory by 32-bit address, and 16-byte asynchronous copies into it.
 __device__ __forceinline__ float4 lds4(unsigned a) {
