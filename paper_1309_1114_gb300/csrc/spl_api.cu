@@ -94,7 +94,7 @@ struct spl_ctx {
     // (C, T) partials of split tiles
     DevBuf<float2> rec2;
     DevBuf<unsigned long long> pkeys, ptmp, ekeys, etmp;
-    DevBuf<unsigned> rank;
+    DevBuf<unsigned> by_depth;
     DevBuf<int> sort_hist;
     DevBuf<float4> partial;
     DevBuf<int> counts, ovf, full;
@@ -278,7 +278,7 @@ extern "C" int spl_destroy(spl_ctx *c) {
     c->pal.release();
     c->recs.release();
     c->rec2.release(); c->pkeys.release(); c->ptmp.release(); c->ekeys.release();
-    c->etmp.release(); c->rank.release(); c->sort_hist.release(); c->partial.release();
+    c->etmp.release(); c->by_depth.release(); c->sort_hist.release(); c->partial.release();
     c->counts.release(); c->offsets.release(); c->cursor.release();
     c->ovf.release(); c->ctab.release(); c->full.release();
     c->large_ids.release(); c->entries.release(); c->dstats.release();
@@ -629,7 +629,7 @@ static int prepare_views(spl_ctx *c, const spl_camera *cams, int V, float *const
         SPL_TRY(grow(c, c->rec2, recs ? recs : 1));
         SPL_TRY(grow(c, c->pkeys, recs ? recs : 1));
         SPL_TRY(grow(c, c->ptmp, recs ? recs : 1));
-        SPL_TRY(grow(c, c->rank, recs ? recs : 1));
+        SPL_TRY(grow(c, c->by_depth, recs ? recs : 1));
     }
     SPL_TRY(grow(c, c->large_ids, recs ? recs : 1));
     SPL_TRY(grow(c, c->counts, (size_t)NLIST * tiles));
@@ -751,7 +751,8 @@ static void enqueue_lists(spl_ctx *c, const Views &vs, cudaStream_t s) {
     ba.entries = c->entries.p;
     ba.entries_cap = (int64_t)c->entries.cap;
     ba.st = c->dstats.p;
-    const ListArgs la{c->item_offsets.p, c->items.p, (int)c->items.cap, seg_sms(c), c->d_images.p, 0, 0, 0};
+    const ListArgs la{c->item_offsets.p, c->items.p, (int)c->items.cap, seg_sms(c), c->d_images.p,
+                      c->par.mode != SPL_MODE_ABSORB, 0, 0, 0};
     launch_lists(vs, ba, la, !c->accumulate, c->sms, s);
 }
 
@@ -792,9 +793,9 @@ static void enqueue_passes(spl_ctx *c, const Views &vs, bool large_pass, cudaStr
     if (c->par.mode == SPL_MODE_ABSORB) {
         // one view: every entry sits in the medium slots [L_MEDIUM * nt, (L_MEDIUM + 1) * nt]
         const int nt = c->h_fcs[0].ntiles;
-        launch_depth_order(c->recs.p, c->rec2.p, vs.n, c->entries.p, c->offsets.p + L_MEDIUM * nt,
-                           nt, (long long)c->hstats->slot_total, c->pkeys.p, c->ptmp.p,
-                           c->ekeys.p, c->etmp.p, c->rank.p, c->sort_hist.p, c->sms, s);
+        launch_depth_order(vs, c->recs.p, c->rec2.p, c->entries.p, c->offsets.p + L_MEDIUM * nt, nt,
+                           (long long)c->hstats->slot_total, c->pkeys.p, c->ptmp.p, c->ekeys.p,
+                           c->etmp.p, c->by_depth.p, c->sort_hist.p, c->dstats.p, c->sms, s);
         ta.rec2 = c->rec2.p;
         ta.partial = c->partial.p;
         record_event(c, 2, s);

@@ -241,6 +241,7 @@ size_t slot_parts(int tiles);
 
 // Exclusive scan of in[0..m) into out[0..m] (out[m] = total).
 void launch_scan(int m, const int *in, int *out, cudaStream_t s);
+void launch_wide_scan(int m, const int *in, int *out, int *part, cudaStream_t s);
 
 // The tile lists, the work items and (zero) the cleared images.  The caller fills the
 // first five fields of l.
@@ -249,6 +250,7 @@ struct ListArgs {
     WorkItem *items;
     int items_cap, seg_sms;
     float *const *images;
+    bool scatter;                 // fill the lists of points, small and medium particles
     int large_blocks, item_blocks, zero_blocks;
 };
 void launch_lists(const Views &v, BinArgs a, ListArgs l, bool zero, int sms, cudaStream_t s);
@@ -265,11 +267,13 @@ void launch_absorb_pass(const Views &v, const TileArgs &a, const int *item_offse
                         cudaStream_t s);
 int radix_blocks(int64_t n);
 int64_t radix_scratch_ints(int64_t n);
-void launch_depth_order(const Rec *recs, const float2 *rec2, int64_t n, unsigned *entries,
+void launch_depth_order(const Views &vs, const Rec *recs, const float2 *rec2, unsigned *entries,
                         const long long *off, int ntiles, long long total, unsigned long long *pkeys,
-                        unsigned long long *ptmp, unsigned long long *ekeys,
-                        unsigned long long *etmp, unsigned *rank, int *hist, int sms,
-                        cudaStream_t s);
+                        unsigned long long *ptmp, unsigned long long *ekeys, unsigned long long *etmp,
+                        unsigned *by_depth, int *hist, DevStats *st, int sms, cudaStream_t s);
+void launch_depth_entries(const Views &vs, const Rec *recs, const unsigned *by_depth,
+                          unsigned long long *keys, long long total, int *counts, DevStats *st,
+                          cudaStream_t s);
 void launch_epilogue_ea(float *image, int64_t nvals, int sms, cudaStream_t s);
 // FP32 attributes h, I, s into storage layout `store` (SPL_ATTR_* value).
 void launch_encode_attrs(const float *h, const float *I, const float *s, int64_t n, int store,

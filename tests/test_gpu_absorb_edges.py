@@ -40,3 +40,27 @@ def test_one_crowded_tile(rnd, tile, n, scale):
     o = oracle.render(p, scenes.ramp_palette(), cam, par, nthreads=os.cpu_count() or 1)
     B, _ = oracle.ambiguity(p, scenes.ramp_palette(), cam, par)
     assert rel_pixel_error(g, o, B) <= 1e-4
+
+
+# the lists in depth order: one tile (no tile bits), 2^k and 2^k + 1 tiles around the passes of
+# up to eight bits, more than 2^16; particles around a warp's run of 32 and its doubling above
+# 2^21; depths that are all equal or in a few planes keep the index order
+@pytest.mark.parametrize("n,width,height,tile,planes", [
+    (1, 16, 16, 16, 1), (33, 64, 64, 64, 4), (500, 256, 256, 16, 1), (511, 272, 256, 16, 3),
+    (4097, 512, 520, 32, 0), (3000, 4112, 4096, 16, 5), (65 * 32, 100, 37, 32, 2),
+    (2_097_185, 48, 40, 16, 0)])
+def test_lists_in_depth_order(rnd, n, width, height, tile, planes):
+    import torch
+    rng = np.random.default_rng(n)
+    h = 1e-4 if n > 10000 else 0.02 if width < 1000 else 0.002
+    p = {"x": rng.random(n), "y": rng.random(n), "z": rng.random(n), "h": np.full(n, h),
+         "I": np.full(n, 2.0 if n < 10000 else 0.02), "s": rng.random(n)}
+    if planes:
+        p["z"] = np.floor(p["z"] * planes) / planes
+    p = {k: v.astype(np.float32) for k, v in p.items()}
+    cam = scenes.camera(width, height)
+    g = gpu_render(rnd, torch, p, scenes.ramp_palette(), cam, mode=2, tile_px=tile)
+    par = {"mode": 2}
+    o = oracle.render(p, scenes.ramp_palette(), cam, par, nthreads=os.cpu_count() or 1)
+    B, _ = oracle.ambiguity(p, scenes.ramp_palette(), cam, par)
+    assert rel_pixel_error(g, o, B) <= 1e-4
