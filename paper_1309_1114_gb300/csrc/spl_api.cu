@@ -751,8 +751,8 @@ static void enqueue_lists(spl_ctx *c, const Views &vs, cudaStream_t s) {
     ba.entries = c->entries.p;
     ba.entries_cap = (int64_t)c->entries.cap;
     ba.st = c->dstats.p;
-    const ListArgs la{c->item_offsets.p, c->items.p, (int)c->items.cap, seg_sms(c), c->d_images.p,
-                      c->par.mode != SPL_MODE_ABSORB, 0, 0, 0};
+    const ListArgs la{c->item_offsets.p, c->items.p, (int)c->items.cap, seg_sms(c), c->d_images.p, 0, 0, 0,
+                      c->par.mode != SPL_MODE_ABSORB};
     launch_lists(vs, ba, la, !c->accumulate, c->sms, s);
 }
 

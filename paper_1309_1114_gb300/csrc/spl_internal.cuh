@@ -250,8 +250,8 @@ struct ListArgs {
     WorkItem *items;
     int items_cap, seg_sms;
     float *const *images;
-    bool scatter;                 // fill the lists of points, small and medium particles
     int large_blocks, item_blocks, zero_blocks;
+    bool scatter = true;          // fill the lists of points, small and medium particles
 };
 void launch_lists(const Views &v, BinArgs a, ListArgs l, bool zero, int sms, cudaStream_t s);
 void launch_tile_pass(const Views &v, const TileArgs &a, int sms, cudaStream_t s);
