@@ -95,6 +95,7 @@ struct spl_ctx {
     DevBuf<float2> rec2;
     DevBuf<unsigned long long> pkeys, ptmp, ekeys, etmp;
     DevBuf<unsigned> by_depth;
+    DevBuf<float> front;
     DevBuf<int> sort_hist;
     DevBuf<float4> partial;
     DevBuf<int> counts, ovf, full;
@@ -278,7 +279,7 @@ extern "C" int spl_destroy(spl_ctx *c) {
     c->pal.release();
     c->recs.release();
     c->rec2.release(); c->pkeys.release(); c->ptmp.release(); c->ekeys.release();
-    c->etmp.release(); c->by_depth.release(); c->sort_hist.release(); c->partial.release();
+    c->etmp.release(); c->by_depth.release(); c->front.release(); c->sort_hist.release(); c->partial.release();
     c->counts.release(); c->offsets.release(); c->cursor.release();
     c->ovf.release(); c->ctab.release(); c->full.release();
     c->large_ids.release(); c->entries.release(); c->dstats.release();
@@ -798,6 +799,14 @@ static void enqueue_passes(spl_ctx *c, const Views &vs, bool large_pass, cudaStr
                            c->etmp.p, c->by_depth.p, c->sort_hist.p, c->dstats.p, c->sms, s);
         ta.rec2 = c->rec2.p;
         ta.partial = c->partial.p;
+        if (front_pays(c->hstats->item_totals[0], vs.total_tiles, c->sms)) {
+            ta.front = c->front.p;
+            launch_segment_order(ta, c->item_offsets.p, vs.tile, sched ? nullptr : c->cost.p, s);
+            if (!sched) {
+                launch_order_items(c->cost.p, ta.items_cap, c->dstats.p, c->order_hist.p, c->order.p, s);
+                ta.order = c->order.p;
+            }
+        }
         record_event(c, 2, s);
         launch_absorb_pass(vs, ta, c->item_offsets.p, c->sms, s);
         record_event(c, 3, s);
@@ -878,6 +887,7 @@ static int render_views(spl_ctx *c, const spl_camera *cams, int V, float *const 
         SPL_TRY(grow(c, c->etmp, (size_t)(total ? total : 1)));
         SPL_TRY(grow(c, c->sort_hist, (size_t)radix_scratch_ints(m)));
         SPL_TRY(grow(c, c->partial, c->items.cap * (size_t)vs.tile * (size_t)vs.tile));
+        SPL_TRY(grow(c, c->front, c->items.cap * (size_t)(vs.tile == 64 ? 4 : 1)));
     }
     c->last_items = n_tile_items + n_large_items;
     enqueue_passes(c, vs, n_large_items > 0, s);

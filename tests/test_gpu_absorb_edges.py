@@ -64,3 +64,28 @@ def test_lists_in_depth_order(rnd, n, width, height, tile, planes):
     o = oracle.render(p, scenes.ramp_palette(), cam, par, nthreads=os.cpu_count() or 1)
     B, _ = oracle.ambiguity(p, scenes.ramp_palette(), cam, par)
     assert rel_pixel_error(g, o, B) <= 1e-4
+
+
+# more segments than are worked on at a time: those behind opaque ones are left out, tile by tile
+# (and part by part at 64), those behind transparent ones are not; `right` scales A in the
+# right half of the image
+@pytest.mark.parametrize("sched", [0, 1])
+@pytest.mark.parametrize("tile", [16, 32, 64])
+@pytest.mark.parametrize("right", [1.0, 1e-3, 1e-6])
+def test_hidden_segments(rnd, tile, right, sched):
+    import torch
+    n, rng = 620_000, np.random.default_rng(5)
+    p = {k: rng.random(n) for k in ("x", "y", "z", "I")}
+    p["x"], p["y"] = 2 * p["x"] - 0.5, 2 * p["y"] - 0.5       # the whole image is covered
+    p["h"] = rng.uniform(0.01, 0.03, n)
+    p["I"] *= np.where(p["x"] > 0.5, right, 1.0)
+    p["s"] = rng.random(n)
+    p = {k: v.astype(np.float32) for k, v in p.items()}
+    pal = scenes.ramp_palette()
+    cam = scenes.camera(75, 61)
+    g = gpu_render(rnd, torch, p, pal, cam, mode=2, tile_px=tile, sched=sched)
+    par = {"mode": 2}
+    o = oracle.render(p, pal, cam, par, nthreads=os.cpu_count() or 1)
+    B, _ = oracle.ambiguity(p, pal, cam, par)
+    assert rnd.stats()["n_entries"][2] > 1024 * (75 * 61 / tile ** 2 + 500)
+    assert rel_pixel_error(g, o, B) <= 1e-4
