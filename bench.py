@@ -628,6 +628,10 @@ def run_ours(args, wl):
                 "work": {"point_deposits": work[0], "small_pairs": work[1],
                          "medium_pairs": work[2], "large_pairs": work[3],
                          "flops_per_pair": per_pair}}
+    if absorbing:
+        # segments behind opaque ones are left out by the kernel
+        roofline["work"]["counted"] = "every covered pair of the frame, hidden ones included: no rate is given"
+        roofline["achieved"] = roofline["frac"] = None
     schedulers = None
     if wl.get("sched"):
         # the same frame with each scheduler (CUDA-event frame times, 5 frames each)

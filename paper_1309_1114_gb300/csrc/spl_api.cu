@@ -1,7 +1,8 @@
 // spl_api.cu -- the C ABI (include/splotch.h): context, particle storage,
 // camera / colour map / parameters, and the per-frame pipeline
-//   raster+count -> count large -> scan -> [sync: size lists] -> scatter ->
-//   tile pass -> large pass -> (E=A epilogue)
+//   setup -> raster+count -> count large -> offsets and items -> [sync: size lists] ->
+//   lists -> tile pass -> large pass -> (E=A epilogue)
+// or, in the absorption mode, lists in depth order -> absorption pass -> composition,
 // all on one stream.
 #include <atomic>
 #include <cmath>
@@ -90,8 +91,8 @@ struct spl_ctx {
     spl_params par{};
     // scratch
     DevBuf<Rec> recs;
-    // absorption mode: (A, depth key) per record, the depth-order sort, and the
-    // (C, T) partials of split tiles
+    // absorption mode: (A, depth key) per record, the depth-order sort, what each
+    // segment lets through, and the (C, T) partials of split tiles
     DevBuf<float2> rec2;
     DevBuf<unsigned long long> pkeys, ptmp, ekeys, etmp;
     DevBuf<unsigned> by_depth;

@@ -1,7 +1,8 @@
 // spl_raster.cu -- rasterisation (Sec. 2 "Processing and Rasterization",
 // Sec. 4 one-thread-per-particle) and binning of particles into tile lists
 // (the data organisation of Sec. 4, built with counts, a scan and a scatter
-// instead of a radix sort by tile index).
+// instead of a radix sort by tile index; the absorption mode, whose lists are in
+// depth order, sorts them by tile).
 #include <cstddef>
 
 #include "spl_geom.cuh"
@@ -189,7 +190,7 @@ __device__ __forceinline__ int raster_one(const FrameConst &fc, const float *spa
 // Tile footprint of one rasterised particle for the point / small / medium
 // lists: a box of tiles [tx0, tx0 + bw) x [ty0, ty0 + nbox / bw) (nbox = 0:
 // no entry); disc = 1 when a tile of the box must also be reached by the disc.
-// Large particles are handled by large_tiles_kernel.  In the absorption mode
+// Large particles are handled by large_tiles.  In the absorption mode
 // points join the medium list, so that a tile's particles form one list that
 // can be ordered by depth.
 struct TileFoot { int list, tx0, ty0, bw, nbox, disc; float reach2; };

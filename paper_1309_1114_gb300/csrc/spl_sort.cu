@@ -2,7 +2,7 @@
 // form (Eq. 1 with E_p != A_p), where the particles a ray crosses must be
 // taken in depth order (the sort step of Sec. 4 with a depth key).
 //
-// A stable least-significant-digit radix sort of 64-bit keys, 8-bit digits:
+// A stable least-significant-digit radix sort of 64-bit keys, digits of up to 8 bits:
 // per pass, every block of kSortTile keys counts its digits (hist[digit][block]),
 // one exclusive scan over the digit-major table gives every (digit, block) its
 // output base, and every block scatters its keys in their original order.
@@ -21,9 +21,8 @@ namespace spl {
 
 constexpr int kSortThreads = 256;
 // keys per thread: 8 keep the scatter at 48 registers and 5 CTAs per SM
-// without spills (16 took 99 registers, 2 CTAs per SM; the scatter and depth
-// sort of the clustered 10M frame went from 4.64 to 3.77 ms, same result; 4
-// keys per thread at 6 or 8 CTAs per SM: 4.12 and 3.84 ms)
+// without spills (four passes over 10M keys and five over 30M: 3.77 ms; 16 keys, 99
+// registers and 2 CTAs per SM: 4.64; 4 keys at 6 or 8 CTAs per SM: 4.12 and 3.84)
 constexpr int kSortItems = 8;
 constexpr int kSortTile = kSortThreads * kSortItems;            // keys per block
 
