@@ -957,7 +957,9 @@ __device__ __forceinline__ void scatter_chunk(const Views &vs, const BinArgs &a,
 
 // Everything that follows the offsets, in one launch, by the block's number: the large
 // lists, the work items and the cleared images are a few blocks' work beside the
-// scatter, and each was a launch of its own.
+// scatter, and each was a launch of its own.  The images' blocks come last, so that small
+// frames' chunks all start at once and the cleared pixels are still in L2 for the tile pass
+// (200k particles: lists 29 -> 27 us; 1.3M: frame 1.089 -> 1.085 ms).
 __global__ void __launch_bounds__(256, 6) lists_kernel(Views vs, BinArgs a, ListArgs l) {
     extern __shared__ long long lists_smem[];
     int b = blockIdx.x;
@@ -966,22 +968,24 @@ __global__ void __launch_bounds__(256, 6) lists_kernel(Views vs, BinArgs a, List
         return;
     }
     b -= l.large_blocks;
+    const int fill = (int)gridDim.x - l.large_blocks - l.item_blocks - l.zero_blocks;
+    if (b < fill) {
+        scatter_chunk(vs, a, b, lists_smem);
+        return;
+    }
+    b -= fill;
     if (b < l.item_blocks) {
         fill_items(vs, a.offsets, l.item_offsets, l.items, l.items_cap, a.st, l.seg_sms, b, l.item_blocks);
         return;
     }
     b -= l.item_blocks;
-    if (b < l.zero_blocks) {
-        for (int v = 0; v < vs.nviews; ++v) {
-            const int64_t n = (int64_t)3 * vs.fcs[v].width * vs.fcs[v].height;
-            float *img = l.images[v];
-            for (int64_t i = (int64_t)b * blockDim.x + threadIdx.x; i < n;
-                 i += (int64_t)l.zero_blocks * blockDim.x)
-                img[i] = 0.f;
-        }
-        return;
+    for (int v = 0; v < vs.nviews; ++v) {
+        const int64_t n = (int64_t)3 * vs.fcs[v].width * vs.fcs[v].height;
+        float *img = l.images[v];
+        for (int64_t i = (int64_t)b * blockDim.x + threadIdx.x; i < n;
+             i += (int64_t)l.zero_blocks * blockDim.x)
+            img[i] = 0.f;
     }
-    scatter_chunk(vs, a, b - l.zero_blocks, lists_smem);
 }
 
 void launch_lists(const Views &vs, BinArgs a, ListArgs l, bool zero, int sms, cudaStream_t s) {
