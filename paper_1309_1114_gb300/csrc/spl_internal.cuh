@@ -123,17 +123,21 @@ struct Segs {
 constexpr int kHashBits = 11;
 constexpr int kHash = 1 << kHashBits;
 constexpr int kChunk = 2048;
-// Sets that give the SMs less than kFewChunks CTAs of that size go through quarter
-// chunks with quarter tables: a CTA takes its chunk 256 particles at a time, so that a
-// longer chunk is a longer chain (200k particles: raster 0.032 -> 0.022, lists 0.043 ->
-// 0.029 ms; 1.3M: 0.107 -> 0.087, 0.163 -> 0.113). On larger sets the four times as many
-// tables cost more (10M: raster 0.369 -> 0.588 ms; the two meet near 3M).
+// Sets that give the SMs less than kFewChunks CTAs of that size go through half chunks
+// with half tables, and those that give them less than kQuarter through quarters: a CTA takes
+// its chunk 256 particles at a time, so that a longer chunk is a longer chain (200k
+// particles: raster 0.032 -> 0.022, lists 0.043 -> 0.029 ms in quarters; 1.3M clustered: 0.107 ->
+// 0.079, 0.163 -> 0.098 in halves), but every table adds each of its slots to the global counts
+// (10M: raster 0.369 ms, 0.588 in quarters; the two meet near 3M).  1.3M in quarters and
+// halves: clustered frame 1.084 and 1.097 ms, uniform 0.781 and 0.676; 1.7M clustered 0.338 and 0.312.
 struct BinShape {
     int chunk, hash_bits;
 };
-constexpr int kFewChunks = 10;
+constexpr int kFewChunks = 10, kQuarter = 3;
 __host__ __device__ inline BinShape bin_shape(int64_t n, int sms) {
-    return n < (int64_t)sms * kFewChunks * kChunk ? BinShape{kChunk / 4, kHashBits - 2} : BinShape{kChunk, kHashBits};
+    if (n < (int64_t)sms * kQuarter * kChunk) return BinShape{kChunk / 4, kHashBits - 2};
+    return n < (int64_t)sms * kFewChunks * kChunk ? BinShape{kChunk / 2, kHashBits - 1}
+                                                  : BinShape{kChunk, kHashBits};
 }
 __host__ __device__ constexpr int64_t ctab_entries(int64_t n, int nviews) {
     return ((n + kChunk - 1) / kChunk > 0 ? (n + kChunk - 1) / kChunk : 1) *

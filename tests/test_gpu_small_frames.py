@@ -88,3 +88,18 @@ def test_replayed_lists_that_outgrow_their_buffers(grow):
             assert rel_pixel_error(im.cpu().numpy().astype(np.float64), o, B) <= 1e-4
     finally:
         r.close()
+
+
+@pytest.mark.parametrize("chunks", [3, 10])      # 2048-particle chunks per SM where the binning
+@pytest.mark.parametrize("off", [-1, 0])         # goes from quarter to half chunks, and to whole ones
+def test_chunk_sizes_meet(rnd, chunks, off):
+    import torch
+    n = torch.cuda.get_device_properties(0).multi_processor_count * chunks * 2048 + off
+    rng = np.random.default_rng(chunks)
+    p = {k: rng.random(n, dtype=np.float32) for k in ("x", "y", "z", "I", "s")}
+    p["h"] = np.exp(rng.uniform(-9.0, -6.0, n)).astype(np.float32)
+    pal, cam = scenes.ramp_palette(), scenes.camera(400, 300)
+    o = oracle.render(p, pal, cam, {}, nthreads=os.cpu_count() or 1)
+    B, _ = oracle.ambiguity(p, pal, cam, {})
+    g = gpu_render(rnd, torch, p, pal, cam, tile_px=16)
+    assert rel_pixel_error(g, o, B) <= 1e-4
