@@ -772,6 +772,14 @@ static void enqueue_passes(spl_ctx *c, const Views &vs, bool large_pass, cudaStr
     ta.images = c->d_images.p;
     ta.st = c->dstats.p;
     ta.accumulate = c->accumulate ? 1 : 0;
+    if (c->par.mode == SPL_MODE_ABSORB) {
+        // the depth order writes the lists, which the features read.  One view: every entry
+        // sits in the medium slots [L_MEDIUM * nt, (L_MEDIUM + 1) * nt]
+        const int nt = c->h_fcs[0].ntiles;
+        launch_depth_order(vs, c->recs.p, c->rec2.p, c->entries.p, c->offsets.p + L_MEDIUM * nt, nt,
+                           (long long)c->hstats->slot_total, c->pkeys.p, c->ptmp.p, c->ekeys.p,
+                           c->etmp.p, c->by_depth.p, c->sort_hist.p, c->dstats.p, c->sms, s);
+    }
     // scheduling: per-item features, predicted cost, longest first
     const bool sched = c->par.sched != SPL_SCHED_NONE;
     const float *theta = c->par.sched == SPL_SCHED_MLP && c->have_model ? c->theta.p : nullptr;
@@ -793,11 +801,6 @@ static void enqueue_passes(spl_ctx *c, const Views &vs, bool large_pass, cudaStr
         cudaMemsetAsync(ta.item_cycles, 0, sizeof(long long) * c->item_cycles.cap, s);
     }
     if (c->par.mode == SPL_MODE_ABSORB) {
-        // one view: every entry sits in the medium slots [L_MEDIUM * nt, (L_MEDIUM + 1) * nt]
-        const int nt = c->h_fcs[0].ntiles;
-        launch_depth_order(vs, c->recs.p, c->rec2.p, c->entries.p, c->offsets.p + L_MEDIUM * nt, nt,
-                           (long long)c->hstats->slot_total, c->pkeys.p, c->ptmp.p, c->ekeys.p,
-                           c->etmp.p, c->by_depth.p, c->sort_hist.p, c->dstats.p, c->sms, s);
         ta.rec2 = c->rec2.p;
         ta.partial = c->partial.p;
         if (front_pays(c->hstats->item_totals[0], vs.total_tiles, c->sms)) {
