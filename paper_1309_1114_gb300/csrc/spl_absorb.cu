@@ -62,14 +62,14 @@ __device__ __forceinline__ float lds1(unsigned a) {
     return v;
 }
 
-// Tabulate the particle (r0, r1, A) into the block tab: thread q of its four fills column
+// Tabulate the particle (r0, r1, A), A > 0, into the block tab: thread q of its four fills column
 // pairs and row pairs q, q + 4, ....
 template <int W>
 __device__ __forceinline__ void absorb_tabulate(float4 r0, float4 r1, float A, bool point, int x0, int y0,
                                                 unsigned tab, int q) {
     using Q = Absorb<W>;
     if (q == 0) {
-        const float inv = A > 0.f ? 1.f / A : 0.f;
+        const float inv = 1.f / A;
         const float e0 = r1.y * inv, e1 = r1.z * inv, e2 = r1.w * inv;
         sts2x2(tab + Q::SRC, pack2(e0, e0), pack2(e1, e1));
         sts2x2(tab + Q::SRC + 16, pack2(e2, e2), pack2(A, 0.f));
@@ -289,6 +289,9 @@ __global__ void __launch_bounds__(kTileThreads, kAbsorbCtas) absorb_kernel(Views
                              (int)((long long)n_ent * (rp + 1) / Q::RANGES);
                 const float4 r0 = lds4(st + p * 16), r1 = lds4(st + P * 16 + p * 16);
                 const float A = lds1(st + P * 32 + p * 4);
+                // a particle with A <= 0 neither emits nor absorbs.  (A range starts at T = 1: those of
+                // A < 0, last in the list, would raise T past the largest float there.)
+                valid = valid && A > 0.f;
                 // the blocks in row q of blocks that the particle reaches (a point: its
                 // pixel's; a disc, with a margin, their pixel centres), as in the additive pass
                 const bool point = r1.x <= r_sml2;
