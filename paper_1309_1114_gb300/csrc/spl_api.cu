@@ -1312,10 +1312,12 @@ extern "C" int spl_mlp_loss_grad(const float *d_theta, const float *d_x, const f
     }
     cudaStream_t s = (cudaStream_t)stream;
     launch_mlp_loss_grad(d_theta, d_x, d_t, B, work, d_grad, d_loss, s);
-    int rc = cuda_status(cudaGetLastError());
-    if (rc == SPL_OK) rc = cuda_status(cudaStreamSynchronize(s));
+    // wait also when an error is reported, which may be one that earlier work left: the
+    // kernels are queued all the same, and the slot goes to the next call
+    const int launched = cuda_status(cudaGetLastError());
+    const int waited = cuda_status(cudaStreamSynchronize(s));
     if (own) cudaFree(own);
-    return rc;
+    return launched != SPL_OK ? launched : waited;
 }
 
 extern "C" int spl_mlp_adam(float *d_theta, const float *d_grad, float *d_m, float *d_v, int64_t np,
