@@ -991,12 +991,14 @@ __global__ void __launch_bounds__(256, 6) lists_kernel(Views vs, BinArgs a, List
 void launch_lists(const Views &vs, BinArgs a, ListArgs l, bool zero, int sms, cudaStream_t s) {
     a.shape = bin_shape(vs.n, sms);
     const int64_t chunks = vs.n > 0 && l.scatter ? (vs.n + a.shape.chunk - 1) / a.shape.chunk : 0;
+    // 8 to 32 KB by the set's size, beside 9 KB of static shared memory: within the 48 KB that need
+    // no attribute.  (The attribute is the kernel's, not the launch's: a launch of another
+    // thread that set it for a smaller set made this one fail.)
     const size_t smem = ((size_t)1 << a.shape.hash_bits) * (sizeof(long long) + 2 * sizeof(int));
     l.large_blocks = vs.n > 0 ? sms * 2 : 0;
     const int warps = (vs.total_tiles + 7) / 8;     // 8 warps of 256 threads, a warp per tile
     l.item_blocks = warps < sms * 4 ? warps : sms * 4;
     l.zero_blocks = zero ? sms * 2 : 0;
-    cudaFuncSetAttribute(lists_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     const int64_t blocks = l.large_blocks + l.item_blocks + l.zero_blocks + chunks;
     lists_kernel<<<(unsigned)blocks, 256, smem, s>>>(vs, a, l);
     ++g_launches;
