@@ -300,7 +300,8 @@ int spl_count_work(spl_ctx *ctx, int64_t out[4]);
 int spl_set_model(spl_ctx *ctx, const float *theta, const float *heur);
 
 /* With recording on, every render also stores each work item's features and
- * the SM clock cycles its CTA spent on it (clock64 difference). */
+ * the SM clock cycles its CTA spent on it (clock64 difference; the absorption
+ * mode does not count them: d_logc is 0 there). */
 int spl_set_recording(spl_ctx *ctx, int32_t enable);
 
 /* Copy the last render's samples (at most cap) into DEVICE buffers:

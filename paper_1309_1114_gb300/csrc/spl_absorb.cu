@@ -26,11 +26,11 @@ namespace spl {
 // the other: the two quarters of a block (and the four warps that share a pair of blocks at
 // W = 16) work on different ranges, whose (C, T) are composed at the end.
 //
-// What bounds it: issue and latency -- 24 packed operations per lane and step beside the
+// What bounds it: issue and latency -- 14 packed operations per pixel pair and step beside the
 // loads, and each pixel's T is a chain.  One particle per warp step over a 16 x 8 band, a
 // lane 2 x 2 pixels, records fetched between two barriers, took 9.48 ms on the
 // clustered 10M / 1024^2 frame (covered to 54 %; 8 x 8 blocks to 65 %); this takes
-// 8.13 ms (1.17 since hidden segments are left out, below).
+// 8.13 ms (1.24 since hidden segments are left out, below).
 template <int W>
 struct Absorb {
     static constexpr int P = 64;                   // particles per batch
@@ -177,12 +177,14 @@ __device__ __forceinline__ float4 compose(float4 front, float4 back) {
 // A segment behind others is left out once nothing in it can show: a.front holds, per
 // segment (and part of a 64-pixel tile), log2 of the largest transmittance of its
 // pixels, 0 until it is done, and kHidden when it is left out.  Where the segments in front
-// come to less than kOpaque, every pixel's transmittance there is below half of the
-// smallest float: composed, it is 0, and so is what the segment would add.  Whichever of
+// come to less than kOpaque, the product of a pixel's transmittances there is below 2^-160:
+// composed in FP32 it is 0 or, under factors above 1/2, stays at the smallest subnormal, so
+// that the segment would add at most 2^-149 of its colour.  Whichever of
 // the segments in front are done by then, only those count, so that the order of the items
 // is free; they are taken by segment number (segment_order_kernel), so that
 // the front ones of every tile are done first.  Clustered 10M / 1024^2, 29 segments per
-// tile: 8.13 -> 1.17 ms with the order and the composition.
+// tile: 8.13 -> 1.17 ms with the order and the composition (1.24 since the polynomial of
+// 1 - exp(-tau) has a term more).
 constexpr float kOpaque = -160.f, kHidden = -1e30f;
 
 template <int T>

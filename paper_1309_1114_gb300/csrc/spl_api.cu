@@ -1021,9 +1021,10 @@ extern "C" int spl_render_stream(spl_ctx *c, const spl_particles *p, int64_t chu
         rc = render_views(c, &c->cam, 1, &d_image, s);
         if (rc != SPL_OK) break;
         rc = cuda_status(cudaEventRecord(c->consumed[b], s));
-        // the next chunk's copy starts once this chunk's binning is done (render_views
-        // has synchronised after it), so that it overlaps the scatter and tile pass
-        // and does not queue the small per-chunk uploads behind a large copy
+        // the next chunk's copy starts once this chunk's binning is done (render_views has
+        // waited for its counts) and overlaps the lists and the tile pass.  (A chunk's constants
+        // travel as launch arguments and its buffers are read by the raster alone, so that the copy
+        // could start earlier; that has not been measured.)
         if (rc == SPL_OK && k + 1 < nchunks) {
             const int64_t nf = first + chunk;
             rc = copy_chunk(c, p, nf, p->n - nf < chunk ? p->n - nf : chunk, b ^ 1);

@@ -118,12 +118,12 @@ __device__ __forceinline__ void warp_points(const TileArgs &a, bool valid, float
 // 4 x 2 pixels of its block.  The two quarters of a block are added at the end of
 // the item.
 //
-// What bounds it: the shared-memory data pipe (77 % of its peak on the clustered
-// 10M / 1024^2 frame; issue slots 65 %, FMA pipe 55 %).  One particle per warp step
+// What bounds it: the shared-memory data pipe (76 % of its peak on the clustered
+// 10M / 1024^2 frame; issue slots 63 %, FMA pipe 58 %).  One particle per warp step
 // over a 16 x 8 band, a lane 2 x 2 pixels, took 8 wavefronts per 128 pixels at 54 %
-// covered pixels: 34.6 wavefronts and 124 instructions per list entry, the pipe at 82 %.
+// covered pixels: 28.7 shared-load wavefronts and 128 instructions per list entry, the pipe at 81 %.
 // 8 x 8 blocks are covered to 65 %, and a lane's eight pixels share its four 16-byte loads
-// (12 wavefronts per 256 pixels): 28.5 wavefronts and 108 instructions.  Tile pass of that
+// (12 wavefronts per 256 pixels): 20.5 wavefronts and 102 instructions.  Tile pass of that
 // frame 4.58 -> 3.84 ms.  Also measured there: a lane 4 x 4 pixels of a 16 x 8 band
 // (fewest wavefronts, but 48 accumulators leave 16 warps per SM: 4.65), the same with
 // producer warps and an mbarrier ring (4.50), 3 CTAs per SM (4.55), the clip as
