@@ -1067,6 +1067,7 @@ static unsigned long long batch_key(const spl_ctx *c, const spl_camera *cams, in
     mix(&c->have_rgb, sizeof(c->have_rgb));
     mix(&c->h_log2_min, sizeof(c->h_log2_min));
     mix(&c->npal, sizeof(c->npal));
+    mix(&c->recording, sizeof(c->recording));      // (launches of the graph, and its segments)
     mix(&c->buf_gen, sizeof(c->buf_gen));
     return h;
 }
